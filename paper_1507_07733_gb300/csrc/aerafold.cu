@@ -338,6 +338,20 @@ cudaError_t set_unfold_smem_limit(size_t bytes) {
   return e;
 }
 
+// The station kernel's shared memory, and its SMs' split between L1 and shared memory set for the
+// largest share: the unfold kernel's first CTAs start beside it and build their first inverse,
+// which an SM set up for the station kernel's own 18-72 KB refuses (on a scan of 124 x 64 pairs at
+// 2048 samples three quarters of them started 4-6 us after it, now 1 us).
+template <int N_>
+cudaError_t set_station_limits() {
+  cudaError_t e = cudaFuncSetAttribute(station_spectrum_kernel<N_>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       static_cast<int>(SpectrumSmem<N_>::TOTAL));
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(station_spectrum_kernel<N_>, cudaFuncAttributePreferredSharedMemoryCarveout,
+                             cudaSharedmemCarveoutMaxShared);
+  return e;
+}
+
 template <int N_>
 ar_status unfold_cfg(ar_ctx* ctx, int n_f, KernelCfg** out) {
   std::lock_guard<std::recursive_mutex> lk(ctx->mu);
@@ -359,8 +373,7 @@ ar_status unfold_cfg(ar_ctx* ctx, int n_f, KernelCfg** out) {
     kc.smem = UnfoldSmem<N_>::total(n_f, kc.slab_direct != 0);
     if (per_sm < 1) return fail(ctx, AR_ERR_CUDA, "unfold kernel N=%d does not fit an SM (smem %zu)", N_, kc.smem);
     kc.grid = per_sm * ctx->num_sms;
-    AR_CUDA(ctx, cudaFuncSetAttribute(station_spectrum_kernel<N_>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      static_cast<int>(SpectrumSmem<N_>::TOTAL)));
+    AR_CUDA(ctx, set_station_limits<N_>());
     it = ctx->unfold_cfg.emplace(key, kc).first;
   }
   *out = &it->second;
@@ -1383,17 +1396,15 @@ ar_status ar_batch_create(ar_ctx* ctx, const ar_batch_limits* lim, ar_batch** ou
              : c == 1 ? UnfoldSmem<2048>::total(lim->max_n_freq, direct)
                       : UnfoldSmem<4096>::total(lim->max_n_freq, direct);
     };
-    const size_t sp_smem = c == 0 ? SpectrumSmem<1024>::TOTAL : c == 1 ? SpectrumSmem<2048>::TOTAL : SpectrumSmem<4096>::TOTAL;
-    const void* sfn = c == 0 ? reinterpret_cast<const void*>(station_spectrum_kernel<1024>)
-                      : c == 1 ? reinterpret_cast<const void*>(station_spectrum_kernel<2048>)
-                               : reinterpret_cast<const void*>(station_spectrum_kernel<4096>);
     const size_t smem_max = c == 0 ? UnfoldSmem<1024>::total(kMaxFreqNodes)
                             : c == 1 ? UnfoldSmem<2048>::total(kMaxFreqNodes)
                                      : UnfoldSmem<4096>::total(kMaxFreqNodes);
     if ((e = c == 0   ? set_unfold_smem_limit<1024>(smem_max)
              : c == 1 ? set_unfold_smem_limit<2048>(smem_max)
                       : set_unfold_smem_limit<4096>(smem_max)) != cudaSuccess ||
-        (e = cudaFuncSetAttribute(sfn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(sp_smem))) != cudaSuccess ||
+        (e = c == 0   ? set_station_limits<1024>()
+             : c == 1 ? set_station_limits<2048>()
+                      : set_station_limits<4096>()) != cudaSuccess ||
         (e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b->max_ctas_per_sm[c], fn, threads, smem_of(false))) !=
             cudaSuccess)
       return cleanup(fail(ctx, AR_ERR_CUDA, "kernel set-up failed: %s", cudaGetErrorString(e)));
@@ -2126,12 +2137,9 @@ ar_status noalloc_setup(int dev, NoAllocDevice** out) {
     AR_NA_CUDA(cudaGetSymbolAddress(&p, g_noalloc_scratch));
     AR_NA_CUDA(upload_pretwiddles());
     AR_NA_CUDA(cudaDeviceGetAttribute(&d.num_sms, cudaDevAttrMultiProcessorCount, dev));
-    const size_t sp1 = SpectrumSmem<1024>::TOTAL;
-    const size_t sp2 = SpectrumSmem<2048>::TOTAL;
-    const size_t sp4 = SpectrumSmem<4096>::TOTAL;
-    AR_NA_CUDA(cudaFuncSetAttribute(station_spectrum_kernel<1024>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(sp1)));
-    AR_NA_CUDA(cudaFuncSetAttribute(station_spectrum_kernel<2048>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(sp2)));
-    AR_NA_CUDA(cudaFuncSetAttribute(station_spectrum_kernel<4096>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(sp4)));
+    AR_NA_CUDA(set_station_limits<1024>());
+    AR_NA_CUDA(set_station_limits<2048>());
+    AR_NA_CUDA(set_station_limits<4096>());
     AR_NA_CUDA(set_unfold_smem_limit<1024>(UnfoldSmem<1024>::total(kMaxFreqNodes)));
     AR_NA_CUDA(set_unfold_smem_limit<2048>(UnfoldSmem<2048>::total(kMaxFreqNodes)));
     AR_NA_CUDA(set_unfold_smem_limit<4096>(UnfoldSmem<4096>::total(kMaxFreqNodes)));
