@@ -249,6 +249,18 @@ struct PathParams {
   EventDesc ev0;
 };
 
+// a / b and a mod b of a count a >= 0 (a 64-bit division takes several times a 32-bit one)
+__device__ __forceinline__ void divide(long long a, int b, long long* quot, long long* rem) {
+  if (a <= 0x7fffffffll) {
+    const int x = static_cast<int>(a);
+    *quot = x / b;
+    *rem = x % b;
+  } else {
+    *quot = a / b;
+    *rem = a % b;
+  }
+}
+
 // index of the event whose [begin, begin + count) range holds x (events sorted by begin)
 template <typename F>
 __device__ __forceinline__ int find_event(int n, long long x, F begin_of) {
@@ -379,13 +391,13 @@ __global__ void __launch_bounds__(SpectrumSmem<N_>::BLOCK) station_spectrum_kern
   if (tid >= T) {
     if (ev->dir_pre) {
       // the previous kernel in the stream may still read the entries: wait before writing.
-      // Ten direction slots of three lanes (see precompute_direction); lanes 30, 31 idle.
+      // Eight direction slots of four lanes (see precompute_direction).
       if (prm.wait_prior) pdl_wait_prior();
-      const int lane = tid - T, slot = lane / 3, part = lane % 3;
+      const int lane = tid - T, slot = lane >> 2, part = lane & 3;
       const int S = ev->n_st, D = ev->n_dir;
-      for (int base = s; base < D; base += 10 * S) {   // warp-uniform trip count
+      for (int base = s; base < D; base += 8 * S) {   // warp-uniform trip count
         const int d = base + S * slot;
-        precompute_direction(*ev, d, part, slot < 10 && d < D);
+        precompute_direction(*ev, d, part, d < D);
       }
     }
     continue;
@@ -475,33 +487,49 @@ struct DirPre {
   double pad;
 };
 
-// Direction -> pattern cell (FP64, no fused multiply-adds) -> FP32 bilinear weights.
-__device__ __forceinline__ DirInfo direction_cell(const PatternRef& p, double zen, double az) {
+// Direction -> pattern cell (FP64, no fused multiply-adds) -> FP32 bilinear weights, in two
+// halves that different lanes can form (FP64 is slow here: a chain of two divisions and one of
+// one take less time side by side).
+//
+// The azimuth's position in the table's steps, reduced to [0, n_az]; false if it has none. An
+// azimuth has a place when it is finite and less than 2^52 azimuth steps from az0 (beyond, one
+// FP64 unit is a whole step). Below that bound the remainder modulo n_az lands in [0, n_az]; the
+// range test keeps every slab index in bounds.
+__device__ __forceinline__ bool azimuth_position(const PatternRef& p, double az, double* ua_out) {
+  double ua = 0.0;
+  bool ok = isfinite(az);
+  if (ok) {
+    ua = __ddiv_rn(__dsub_rn(az, p.az0), p.daz);
+    ok = fabs(ua) < 0x1p52;
+  }
+  if (ok) {
+    ua = __dsub_rn(ua, __dmul_rn(double(p.n_az), floor(__ddiv_rn(ua, double(p.n_az)))));
+    ok = ua >= 0.0 && ua <= double(p.n_az);
+  }
+  *ua_out = ua;
+  return ok;
+}
+// The zenith's position, clamped to [0, n_zen - 1] (*clamped); false if it is not finite.
+__device__ __forceinline__ bool zenith_position(const PatternRef& p, double zen, double* uz_out, bool* clamped) {
+  double uz = __ddiv_rn(__dsub_rn(zen, p.zen0), p.dzen);
+  *clamped = false;
+  if (uz < 0.0) { uz = 0.0; *clamped = true; }
+  if (uz > double(p.n_zen - 1)) { uz = double(p.n_zen - 1); *clamped = true; }
+  *uz_out = uz;
+  return isfinite(zen);
+}
+__device__ __forceinline__ DirInfo cell_of_positions(const PatternRef& p, bool has_cell, double uz, bool clamped,
+                                                     double ua) {
   DirInfo di;
   di.st = 0;
   di.pat = -1;
-  // A direction has a cell when it is finite and its azimuth lies less than 2^52 azimuth
-  // steps from az0 (beyond, one FP64 unit is a whole step). Below that bound the remainder
-  // modulo n_az lands in [0, n_az]; the range test keeps every slab index in bounds.
-  double ua = 0.0;
-  bool has_cell = isfinite(zen) && isfinite(az);
-  if (has_cell) {
-    ua = __ddiv_rn(__dsub_rn(az, p.az0), p.daz);
-    has_cell = fabs(ua) < 0x1p52;
-  }
-  if (has_cell) {
-    ua = __dsub_rn(ua, __dmul_rn(double(p.n_az), floor(__ddiv_rn(ua, double(p.n_az)))));
-    has_cell = ua >= 0.0 && ua <= double(p.n_az);
-  }
   if (!has_cell) {   // every output of the direction's pairs is 0
     di.st = kStBadDir;
     di.slab0 = di.slab1 = di.slab2 = di.slab3 = 0;
     di.w[0] = di.w[1] = di.w[2] = di.w[3] = 0.f;
     return di;
   }
-  double uz = __ddiv_rn(__dsub_rn(zen, p.zen0), p.dzen);
-  if (uz < 0.0) { uz = 0.0; di.st |= kStZenClamp; }
-  if (uz > double(p.n_zen - 1)) { uz = double(p.n_zen - 1); di.st |= kStZenClamp; }
+  if (clamped) di.st |= kStZenClamp;
   int iz = static_cast<int>(floor(uz));
   if (iz > p.n_zen - 2) iz = p.n_zen - 2;
   const double tz = __dsub_rn(uz, double(iz));
@@ -519,6 +547,13 @@ __device__ __forceinline__ DirInfo direction_cell(const PatternRef& p, double ze
   di.w[2] = static_cast<float>(__dmul_rn(uz0, ta));
   di.w[3] = static_cast<float>(__dmul_rn(tz, ta));
   return di;
+}
+__device__ __forceinline__ DirInfo direction_cell(const PatternRef& p, double zen, double az) {
+  double ua, uz;
+  bool clamped;
+  const bool ok = azimuth_position(p, az, &ua);
+  const bool zok = zenith_position(p, zen, &uz, &clamped);
+  return cell_of_positions(p, ok && zok, uz, clamped, ua);
 }
 
 // Pre-twiddles of pass 1 for the 1024- and 4096-sample layouts, exp(2 pi i jb r / 4Q) at
@@ -781,20 +816,33 @@ __device__ __forceinline__ DirInfo pair_cell(const EventDesc& ev, int d, int p, 
   return di;
 }
 
-// Part `part` (0, 1, 2) of direction d's entry, by three lanes of one warp in parallel (each
-// part is a chain of slow FP64 operations): 0 the cell, 1 and 2 the sine and cosine of the
-// zenith and of the azimuth, combined into the source vector by lane part 1. valid: d is a
-// direction of the event (all three lanes of a slot agree); the shuffles run regardless.
+// Part `part` (0 .. 3) of direction d's entry, by four lanes of one warp in parallel (each part
+// is a chain of slow FP64 operations): 0 the azimuth's position in the table, 3 the zenith's,
+// combined into the cell by lane part 0; 1 and 2 the sine and cosine of the zenith and of the
+// azimuth, combined into the source vector by lane part 1. valid: d is a direction of the event
+// (all four lanes of a slot agree); the shuffles run regardless.
 __device__ void precompute_direction(const EventDesc& ev, int d, int part, bool valid) {
-  double sv = 0.0, cv = 0.0;
+  double sv = 0.0, cv = 0.0;   // parts 1, 2: sine, cosine; parts 0, 3: the position
+  int flags = 0;               // parts 0, 3: has a position, clamped
+  const bool cell = ev.st_pat == nullptr;
+  const PatternRef pr = pattern_ref(ev, -1);
+  if (valid && (part == 1 || part == 2)) {
+    sincos(ev.dirs[2 * d + (part - 1)], &sv, &cv);
+  } else if (valid && cell && part == 0) {
+    flags = azimuth_position(pr, ev.dirs[2 * d + 1], &sv) ? 1 : 0;
+  } else if (valid && cell) {
+    bool clamped;
+    flags = zenith_position(pr, ev.dirs[2 * d], &sv, &clamped) ? 1 : 0;
+    flags |= clamped ? 2 : 0;
+  }
+  // part 1 (zenith) takes the azimuth's sine and cosine from part 2, part 0 the zenith from part 3
+  const double sa = __shfl_down_sync(0xffffffffu, sv, 1), ca = __shfl_down_sync(0xffffffffu, cv, 1);
+  const double uz = __shfl_down_sync(0xffffffffu, sv, 3);
+  const int zf = __shfl_down_sync(0xffffffffu, flags, 3);
   if (valid && part == 0) {
     DirPre* dp = ev.dir_pre + d;
-    dp->cell = ev.st_pat ? DirInfo{} : pair_cell(ev, d, -1, nullptr);
-  } else if (valid) {
-    sincos(ev.dirs[2 * d + (part - 1)], &sv, &cv);
+    dp->cell = cell ? cell_of_positions(pr, (flags & 1) && (zf & 1), uz, (zf & 2) != 0, sv) : DirInfo{};
   }
-  // part 1 (zenith) takes the azimuth's sine and cosine from part 2, the next lane
-  const double sa = __shfl_down_sync(0xffffffffu, sv, 1), ca = __shfl_down_sync(0xffffffffu, cv, 1);
   if (valid && part == 1) {
     DirPre* dp = ev.dir_pre + d;
     dp->n[0] = __dmul_rn(sv, ca);
@@ -866,6 +914,8 @@ __device__ __forceinline__ bool build_inverse(const EventDesc& ev, int p, const 
   const int tid = threadIdx.x;
   const bool valid = (di.st & (kStBadDir | kStBadPattern)) == 0;
   const PatternRef pr = pattern_ref(ev, p);
+  // the bins' frequency cells, each on its way while the nodes or the bin before are formed
+  int2 next_cell = valid ? __ldg(pr.binf + tid) : make_int2(-1, 0);
   if (valid) {
     const int n_f = pr.n_f;
     const size_t node = static_cast<size_t>(n_f) * 4;
@@ -905,7 +955,8 @@ __device__ __forceinline__ bool build_inverse(const EventDesc& ev, int p, const 
   for (int i = 0; i < NB; ++i) {
     const int j = tid + T * i;
     float4 h0 = make_float4(0.f, 0.f, 0.f, 0.f), h1 = h0;
-    int2 bf = valid ? __ldg(pr.binf + j) : make_int2(-1, 0);
+    int2 bf = next_cell;
+    if (valid && i + 1 < NB) next_cell = __ldg(pr.binf + j + T);
     if (!in_bounds(bf.x < pr.n_f - 1, err)) bf.x = -1;   // a cell past the last node pair
     if (bf.x >= 0) {
       const float tf = __int_as_float(bf.y);
@@ -977,10 +1028,11 @@ __global__ void __launch_bounds__(Layout<N_>::T, Layout<N_>::MIN_CTAS) unfold_ke
   const int n_events = prm.batch ? prm.batch->n_events : 1;
   const long long total_pairs =
       prm.batch ? prm.batch->total_pairs : static_cast<long long>(prm.ev0.n_st) * prm.ev0.n_dir;
-  const long long per = total_pairs / gridDim.x, rem = total_pairs % gridDim.x;
+  long long per, rem;
+  divide(total_pairs, gridDim.x, &per, &rem);
   const long long q0 = blockIdx.x * per + min(static_cast<long long>(blockIdx.x), rem);
-  const long long q1 = q0 + per + (blockIdx.x < rem ? 1 : 0);
-  if (q0 >= q1) {
+  const int n_pairs = static_cast<int>(per) + (blockIdx.x < rem ? 1 : 0);
+  if (n_pairs == 0) {
     if (prm.wait_prior) pdl_wait_prior();
     pdl_launch_dependents();
     return;
@@ -991,9 +1043,10 @@ __global__ void __launch_bounds__(Layout<N_>::T, Layout<N_>::MIN_CTAS) unfold_ke
   // event's station walk, its station s and the station's pattern p (see walk_station)
   int e = e0, d, k;
   {
-    const long long lq = q0 - evs[e0].pair_begin;
-    d = static_cast<int>(lq / evs[e0].n_st);
-    k = static_cast<int>(lq % evs[e0].n_st);
+    long long ld, lk;
+    divide(q0 - evs[e0].pair_begin, evs[e0].n_st, &ld, &lk);
+    d = static_cast<int>(ld);
+    k = static_cast<int>(lk);
   }
   // The station spectra and the walk order come from an earlier kernel; the pattern,
   // directions and station ids do not, unless a skip flag (written by the previous kernel,
@@ -1020,80 +1073,92 @@ __global__ void __launch_bounds__(Layout<N_>::T, Layout<N_>::MIN_CTAS) unfold_ke
   bool pending = slab_staged(evs[e0], p);   // slab copies to wait for before the next build
   __syncthreads();    // barrier initialised, first direction cell visible
 
-  int cur_e = e0 - 1;        // event of the previous pair (none yet)
-  int cur_d = -1;
-  int cur_p = -3;
+  bool new_event = true, new_key = true;   // of the pair at hand
+  int run = 0;               // pairs that follow it in this CTA with the next station of the same key
+  int S = 0;                 // the event's stations, spectra and outputs asked for
+  const float4* spec = nullptr;
+  unsigned wants = 0;
+  constexpr unsigned kTraces = 1, kEnvelope = 2, kFine = 4, kWantSnr = 8, kWalk = 16;
   int pairs_in_dir = 0;
   DirInfo di;
   bool key_sing = false;
   unsigned phase = 0;
   float4 vin[NB];            // the pair's station spectrum at this thread's bins (from L2)
-  const auto load_spec = [&](const EventDesc& x, int st) {
-    if (!in_bounds(st >= 0 && st < x.n_st, prm.err)) {
+  const auto load_spec = [&](const float4* spectra, int n_st, int st) {
+    if (!in_bounds(st >= 0 && st < n_st, prm.err)) {
 #pragma unroll
       for (int i = 0; i < NB; ++i) vin[i] = make_float4(0.f, 0.f, 0.f, 0.f);
       return;
     }
-    const float4* src = x.spec + static_cast<size_t>(st) * M + tid;
+    const float4* src = spectra + static_cast<size_t>(st) * M + tid;
 #pragma unroll
     for (int i = 0; i < NB; ++i) vin[i] = __ldcg(src + T * i);
   };
-  for (long long q = q0; q < q1; ++q) {
-    if (pending) {
-      const unsigned long long limit = prm.test_wait ? kTestWaitLimitNs : kWaitLimitNs;
-      const bool ok = mbar_wait_bounded(bar, phase, limit);
-      if (__syncthreads_or(!ok)) {   // a bulk copy never completed: report, give it one more bounded wait, leave
-        if (tid == 0) {
-          atomicOr(prm.err, kErrTmaTimeout);
-          mbar_wait_bounded(bar, phase, limit);
-          tma_bulk_wait_all();
-        }
-        __syncthreads();
-        return;
-      }
-      phase ^= 1u;
-    }
-    if (e != cur_e) {   // new event: its descriptor into shared memory
-      copy_event(sev, evs + e, tid, T);
-      __syncthreads();
-    }
+  for (int q = 0;; ++q) {
     const EventDesc& ev = *sev;
-    const int S = ev.n_st;
-    // the next pair of this CTA: next station, else next direction, else the next event
-    const bool has_next = q + 1 < q1;
-    int e_next = e, d_next = d, k_next = k + 1;
-    if (k_next == S) {
-      k_next = 0;
-      if (++d_next == ev.n_dir) {
-        d_next = 0;
-        ++e_next;
+    if (new_key) {
+      if (pending) {
+        const unsigned long long limit = prm.test_wait ? kTestWaitLimitNs : kWaitLimitNs;
+        const bool ok = mbar_wait_bounded(bar, phase, limit);
+        if (__syncthreads_or(!ok)) {   // a bulk copy never completed: report, give it one more bounded wait, leave
+          if (tid == 0) {
+            atomicOr(prm.err, kErrTmaTimeout);
+            mbar_wait_bounded(bar, phase, limit);
+            tma_bulk_wait_all();
+          }
+          __syncthreads();
+          return;
+        }
+        phase ^= 1u;
       }
-    }
-    const bool dir_end = !has_next || e_next != e || d_next != d;
-    const EventDesc& evn = e_next != e ? evs[e_next] : ev;
-    // (the walk order may come from the previous kernel: not read before waiting for it)
-    int2 w_next = make_int2(s, p);
-    if (has_next && !(q == q0 && early)) w_next = walk_station(evn, k_next);
-    if (e != cur_e || d != cur_d || p != cur_p) {
-      // new direction or pattern: the inverse of every bin, shared by the key's stations. The
-      // node scratch overlays A: the previous pair's staged outputs must have left it.
+      if (new_event) {   // its descriptor into shared memory
+        copy_event(sev, evs + e, tid, T);
+        __syncthreads();
+        S = ev.n_st;
+        spec = ev.spec;
+        wants = (ev.efield ? kTraces : 0u) | (ev.efield && ev.envelope ? kEnvelope : 0u) |
+                (ev.peak_fine ? kFine : 0u) | (kSnr && ev.snr ? kWantSnr : 0u) | (ev.st_walk ? kWalk : 0u);
+      }
+      // the inverse of every bin, shared by the key's stations. The node scratch overlays A: the
+      // previous pair's staged outputs must have left it.
       di = *sdir;
       if (tid == 0) tma_bulk_wait_read();
       __syncthreads();
       key_sing = build_inverse<N_>(ev, p, di, slab, ev.slab_direct != 0, hn, hinv, prm.err);
-      cur_e = e;
-      cur_d = d;
-      cur_p = p;
-    }
-    if (q == q0) {
-      if (early) {
-        if (prm.wait_prior) pdl_wait_prior();
-        pdl_launch_dependents();
+      run = (wants & kWalk) ? 0 : min(S - 1 - k, n_pairs - 1 - q);
+      if (q == 0) {
+        if (early) {
+          if (prm.wait_prior) pdl_wait_prior();
+          pdl_launch_dependents();
+        }
+        load_spec(spec, S, s);
       }
-      load_spec(ev, s);
-      if (has_next && early) w_next = walk_station(evn, k_next);
     }
-    const int s_next = w_next.x, p_next = w_next.y;
+    // the next pair of this CTA: the run's next station (most pairs: a few instructions, where
+    // looking up the walk for each pair took 80, a tenth of the pair's time), else the next of the
+    // walk, the next direction or the next event
+    bool has_next = true, dir_end = false;
+    int e_next = e, d_next = d;
+    int2 w_next = make_int2(s + 1, p);   // its station and pattern (a walk by pattern: on their way, used below)
+    ++k;
+    if (run > 0) {
+      --run;
+    } else {
+      if (k == S) {
+        k = 0;
+        if (++d_next == ev.n_dir) {
+          d_next = 0;
+          ++e_next;
+        }
+      }
+      has_next = q + 1 < n_pairs;
+      dir_end = !has_next || e_next != e || d_next != d;
+      if (has_next) {
+        if (e_next != e) w_next = walk_station(evs[e_next], k);
+        else if (wants & kWalk) w_next = __ldcg(ev.st_walk + k);
+        else w_next = make_int2(k, p);
+      }
+    }
 
     // ---- 2x2 solve per bin: E = H^-1 V ----
 #pragma unroll
@@ -1111,12 +1176,13 @@ __global__ void __launch_bounds__(Layout<N_>::T, Layout<N_>::MIN_CTAS) unfold_ke
     }
     __syncthreads();   // E complete; the slab buffer is free from here
 
+    const int s_next = w_next.x, p_next = w_next.y;
     const bool next_key = has_next && (dir_end || p_next != p);
     if (tid == 0 && next_key) {   // the next key's direction cell and corner slabs
       fence_proxy_async_smem();
-      issue_key(evn, d_next, p_next, sdir, slab, bar, true, prm.err, prm.test_wait ? 16u : 0u);
+      issue_key(e_next != e ? evs[e_next] : ev, d_next, p_next, sdir, slab, bar, true, prm.err, prm.test_wait ? 16u : 0u);
     }
-    pending = next_key && slab_staged(evn, p_next);
+    pending = next_key && slab_staged(e_next != e ? evs[e_next] : ev, p_next);
 
     // ---- pass 1: Q-point DFTs per (pol, r, ja) ----
     {
@@ -1141,9 +1207,9 @@ __global__ void __launch_bounds__(Layout<N_>::T, Layout<N_>::MIN_CTAS) unfold_ke
     const size_t pair = static_cast<size_t>(d) * S + s;
     // (debug build) the pair lies in the event's outputs; otherwise none of its outputs is written
     const bool pair_ok = in_bounds(e < n_events && d >= 0 && d < ev.n_dir && s >= 0 && s < S, prm.err);
-    const bool traces = ev.efield != nullptr && pair_ok;
-    const bool want_snr = kSnr && ev.snr != nullptr;
-    const bool stage_env = traces || ev.peak_fine != nullptr || want_snr;   // read back by those
+    const bool traces = (wants & kTraces) != 0 && pair_ok;
+    const bool want_snr = kSnr && (wants & kWantSnr) != 0;
+    const bool stage_env = traces || (wants & (kFine | kWantSnr)) != 0;   // read back by those
     float* stage = reinterpret_cast<float*>(reinterpret_cast<unsigned char*>(A) + 16 * M);
     float bv = -1.0f;
     int bi = 0;
@@ -1226,7 +1292,10 @@ __global__ void __launch_bounds__(Layout<N_>::T, Layout<N_>::MIN_CTAS) unfold_ke
         });
       }
     }
-    if (has_next) load_spec(evn, s_next);   // in flight through the pair's end
+    if (has_next) {   // in flight through the pair's end
+      if (e_next == e) load_spec(spec, S, s_next);
+      else load_spec(evs[e_next].spec, evs[e_next].n_st, s_next);
+    }
     // peak: max value, lowest index on ties
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) {
@@ -1240,7 +1309,7 @@ __global__ void __launch_bounds__(Layout<N_>::T, Layout<N_>::MIN_CTAS) unfold_ke
     ++pairs_in_dir;
     if (tid == 0 && traces) {   // the staged E-field (both components) and envelope to global memory
       tma_bulk_s2g(ev.efield + pair * 2 * N, stage, 2 * N * sizeof(float));
-      if (ev.envelope) tma_bulk_s2g(ev.envelope + pair * N, stage + 2 * N, N * sizeof(float));
+      if (wants & kEnvelope) tma_bulk_s2g(ev.envelope + pair * N, stage + 2 * N, N * sizeof(float));
       tma_bulk_commit();
     }
     float snr = 0.f;
@@ -1262,32 +1331,39 @@ __global__ void __launch_bounds__(Layout<N_>::T, Layout<N_>::MIN_CTAS) unfold_ke
       if (bv < 0.f) { bv = 0.f; bi = 0; }
       ev.peak_idx[pair] = bi;
       ev.peak_amp[pair] = bv;   // the peak time is formed with the direction's residual
-      if (ev.peak_fine)
+      if (wants & kFine)
         ev.peak_fine[pair] =
             __dadd_rn(ev.t_start[s], __dmul_rn(__dadd_rn(static_cast<double>(bi), peak_offset(stage + 2 * N, N, bi)),
                                                ev.dt_ns));
       ev.status[pair] = di.st | (key_sing ? kStSingular : 0u);
       if (want_snr) ev.snr[pair] = snr;
     }
-    if (tid == 0 && dir_end) {   // publish this CTA's pairs of direction d; the last CTA does the residual
-      // one acquire-release add: it releases this thread's outputs of the direction (the
-      // only ones the residual reads) and acquires every other CTA's; the barrier below
-      // passes them on to the CTA's other threads
-      *sflag = 0;
-      if (pair_ok) {
-        const unsigned before = atom_add_acq_rel(ev.dir_done + d, static_cast<unsigned>(pairs_in_dir));
-        *sflag = (before + pairs_in_dir == static_cast<unsigned>(S)) ? 1 : 0;
-      }
-    }
     if (dir_end) {
+      // Publish this CTA's pairs of direction d; the last CTA does the residual. One
+      // acquire-release add: it releases thread 0's outputs of the direction (the only ones the
+      // residual reads) and acquires every other CTA's; the barrier passes them on to the
+      // CTA's other threads. A direction that lies in this CTA alone needs the barrier only.
+      if (tid == 0) {
+        *sflag = 0;
+        if (pair_ok) {
+          if (pairs_in_dir == S) {
+            *sflag = 1;
+          } else {
+            const unsigned before = atom_add_acq_rel(ev.dir_done + d, static_cast<unsigned>(pairs_in_dir));
+            *sflag = (before + pairs_in_dir == static_cast<unsigned>(S)) ? 1 : 0;
+          }
+        }
+      }
       pairs_in_dir = 0;
       __syncthreads();
       if (*sflag) direction_residual<T>(ev, d, redd);
     }
+    if (!has_next) break;
     __syncthreads();   // A, reductions and the event copy free for the next pair
+    new_key = next_key;
+    new_event = e_next != e;
     e = e_next;
     d = d_next;
-    k = k_next;
     s = s_next;
     p = p_next;
   }
