@@ -23,6 +23,7 @@
 #include <vector>
 
 #include "../../include/aerafold.h"
+#include "band.h"
 #include "kernels.cuh"
 #include "tc_dft.cuh"
 
@@ -39,8 +40,6 @@ struct NvtxRange {
   NvtxRange& operator=(const NvtxRange&) = delete;
 };
 
-constexpr double kBandLoHz = 30e6;
-constexpr double kBandHiHz = 80e6;
 constexpr double kCMPerNs = 0.299792458;
 
 struct PatternDev {
@@ -127,21 +126,6 @@ ar_status fail(ar_ctx* ctx, ar_status st, const char* fmt, ...) {
                   "%s failed: %s", #call, cudaGetErrorString(e_));                           \
     }                                                                                        \
   } while (0)
-
-// first in-band bin and count; the band is [30, 80] MHz inclusive (same rule as the ABI doc)
-void band_window(int n, double fs, int* k_lo, int* count, int* k_hi) {
-  *k_lo = -1;
-  *count = 0;
-  *k_hi = -1;
-  for (int k = 0; k < n; ++k) {
-    const double f = static_cast<double>(k) * fs / static_cast<double>(n);
-    if (f >= kBandLoHz && f <= kBandHiHz) {
-      if (*k_lo < 0) *k_lo = k;
-      *k_hi = k;
-      ++*count;
-    }
-  }
-}
 
 float2 unit(long t, long n, int sign) {   // exp(sign * 2 pi i t / n), t reduced exactly
   t %= n;
