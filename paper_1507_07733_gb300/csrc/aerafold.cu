@@ -721,7 +721,7 @@ cudaError_t launch_recon(ar_ctx* ctx, const ar_event* ev, int max_iter, double t
   ar_event e1 = *ev;
   e1.n_dirs = 1;
   e1.dirs_rad = st->dir;   // the direction the last fit produced (device memory)
-  PathBuffers b{ctx->spec, ctx->dir_done, ctx->d_err, rs.lt->t1, rs.lt->wn, rs.binf};
+  PathBuffers b{ctx->spec, ctx->dir_done, ctx->d_err, rs.lt->t1, rs.lt->wn, rs.binf, ctx->dir_pre};
   PathParams pp{};
   pp.batch = nullptr;
   pp.err = ctx->d_err;
@@ -733,18 +733,38 @@ cudaError_t launch_recon(ar_ctx* ctx, const ar_event* ev, int max_iter, double t
   const int S = ev->n_stations;
   const double dt_ns = 1e9 / ev->fs_hz;
   const double n_over_c = (ev->refractive_index > 0.0 ? ev->refractive_index : 1.0) / kCMPerNs;
-  cudaError_t e = cudaMemsetAsync(st, 0, sizeof(ReconState), stream);
-  if (e == cudaSuccess && out->history)
-    e = cudaMemsetAsync(out->history, 0xff, sizeof(double) * 2 * (max_iter + 1), stream);   // NaN
-  if (e != cudaSuccess) return e;
-  // the station spectra, once: every iteration unfolds the same traces
+  cudaError_t e;
+  // the station spectra, once: every iteration unfolds the same traces (their direction is not
+  // known yet: its entry comes from the fits)
   PathParams sp = pp;
   sp.skip = nullptr;
+  sp.ev0.dir_pre = nullptr;
   station_spectrum_kernel<N_><<<S, SpectrumSmem<N_>::BLOCK, SpectrumSmem<N_>::TOTAL, stream>>>(sp);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  voltage_peak_kernel<<<S, 256, 0, stream>>>(ev->traces, ev->t_start_ns, ev->n_samples, dt_ns, vidx, vtimes);
-  FitParams fp{ev->pos_m, vtimes, vidx, prev_idx, st, out->history, n_over_c, tol_rad, S, 0};
-  plane_fit_kernel<<<1, 128, 0, stream>>>(fp);
+  // every kernel from here on is launched early behind the previous one and waits for it
+  const int n_history = 2 * (max_iter + 1);
+  if ((e = launch_pdl(voltage_peak_kernel, S, 256, 0, stream, ev->traces, ev->t_start_ns, static_cast<int>(ev->n_samples),
+                      dt_ns, vidx, vtimes, st, out->history, n_history)) != cudaSuccess)
+    return e;
+  FitParams fp{};
+  fp.pos = ev->pos_m;
+  fp.times = vtimes;
+  fp.idx = vidx;
+  fp.prev_idx = prev_idx;
+  fp.st = st;
+  fp.dir_pre = ctx->dir_pre;
+  fp.pattern = PatternRef{pat.table, rs.binf, pat.desc.zen0_rad, pat.desc.dzen_rad, pat.desc.az0_rad,
+                          pat.desc.daz_rad, pat.desc.n_zen, pat.desc.n_az, pat.desc.n_freq, 0};
+  fp.own_pattern = ev->station_pattern ? 0 : 1;
+  fp.direction = out->direction;
+  fp.t0 = out->t0_ns;
+  fp.chi2 = out->chi2;
+  fp.iterations = out->iterations;
+  fp.history = out->history;
+  fp.n_over_c = n_over_c;
+  fp.tol_rad = tol_rad;
+  fp.n_st = S;
+  if ((e = launch_pdl(plane_fit_kernel, 1, 128, 0, stream, fp)) != cudaSuccess) return e;
   for (int it = 1; it <= max_iter; ++it) {
     const size_t smem = UnfoldSmem<N_>::total(pp.ev0.n_f_layout, pp.ev0.slab_direct != 0);
     if ((e = pp.ev0.snr ? launch_pdl(unfold_kernel<N_, true>, std::min(rs.kc->grid, S), L::T, smem, stream, pp)
@@ -754,10 +774,9 @@ cudaError_t launch_recon(ar_ctx* ctx, const ar_event* ev, int max_iter, double t
     fp.times = out->last.peak_time_ns;
     fp.idx = out->last.peak_idx;
     fp.iteration = it;
-    plane_fit_kernel<<<1, 128, 0, stream>>>(fp);
+    if ((e = launch_pdl(plane_fit_kernel, 1, 128, 0, stream, fp)) != cudaSuccess) return e;
   }
-  recon_finish_kernel<<<1, 32, 0, stream>>>(st, out->direction, out->t0_ns, out->chi2, out->iterations);
-  return cudaGetLastError();
+  return cudaSuccess;
 }
 
 }  // namespace

@@ -874,7 +874,7 @@ __device__ __forceinline__ bool slab_staged(const EventDesc& ev, int p) { return
 // For a new (direction, pattern) key (thread 0 only): the key's direction cell into sdir and,
 // when the slabs are staged, the bulk copies of the pattern's four corner slabs, completing
 // the mbarrier's current phase.
-// With pre (after the wait for the station kernel) the event's own pattern's cell is taken
+// With pre (after the wait for the previous kernel) the event's own pattern's cell is taken
 // from the direction's precomputed entry instead of being formed here in FP64.
 __device__ __forceinline__ void issue_key(const EventDesc& ev, int d, int p, DirInfo* sdir, float2* slab,
                                           uint64_t* bar, bool pre = false, unsigned* err = nullptr,
@@ -1068,7 +1068,7 @@ __global__ void __launch_bounds__(Layout<N_>::T, Layout<N_>::MIN_CTAS) unfold_ke
   }
   if (tid == 0) {
     mbar_init(bar, 1);
-    issue_key(evs[e0], d, p, sdir, slab, bar, false, prm.err, prm.test_wait ? 16u : 0u);
+    issue_key(evs[e0], d, p, sdir, slab, bar, !early, prm.err, prm.test_wait ? 16u : 0u);
   }
   bool pending = slab_staged(evs[e0], p);   // slab copies to wait for before the next build
   __syncthreads();    // barrier initialised, first direction cell visible
@@ -1374,11 +1374,8 @@ __global__ void __launch_bounds__(Layout<N_>::T, Layout<N_>::MIN_CTAS) unfold_ke
 
 struct ReconState {        // device memory, one per ar_reconstruct call
   double dir[2];           // direction the next unfold uses (zenith, azimuth)
-  double t0;
-  double chi2;
+  double n[3];             // its unit vector
   int converged;           // set when the direction stops changing (or the fit fails)
-  int iterations;          // unfold iterations whose results were fitted
-  int failed;              // the first fit found no direction
   int pad;
 };
 
@@ -1388,15 +1385,33 @@ struct FitParams {
   const int* idx;          // [S] the sample indices behind those times
   int* prev_idx;           // [S] the indices of the previous fit (updated here)
   ReconState* st;
+  DirPre* dir_pre;         // the direction's cell and vector for the next unfold kernel
+  PatternRef pattern;      // the event's own pattern
+  int own_pattern;         // 0: stations have patterns of their own, no cell is formed
+  // the results of the last fit made: the caller's outputs, written by every fit
+  double* direction;       // [2]
+  double* t0;
+  double* chi2;
+  int* iterations;
   double* history;         // [(max_iter + 1)][2] or null
   double n_over_c, tol_rad;
   int n_st, iteration;     // iteration 0 fits the voltage maxima
 };
 
-// argmax_n v0[n]^2 + v1[n]^2 per station (FP64 squares, lowest index on ties); one CTA per station
+// argmax_n v0[n]^2 + v1[n]^2 per station (FP64 squares, lowest index on ties); one CTA per station.
+// The first CTA also readies the loop's state and history (n_history doubles, or null). Runs
+// beside the station kernel, on which it does not depend, and ends after it, so that what waits for
+// this kernel may use the spectra.
 __global__ void __launch_bounds__(256) voltage_peak_kernel(const float* traces, const double* t_start, int n,
-                                                           double dt_ns, int* idx, double* t_ns) {
+                                                           double dt_ns, int* idx, double* t_ns, ReconState* st,
+                                                           double* history, int n_history) {
   const int s = blockIdx.x, tid = threadIdx.x;
+  pdl_launch_dependents();
+  if (s == 0) {
+    if (tid == 0) *st = ReconState{};
+    if (history)
+      for (int i = tid; i < n_history; i += 256) history[i] = __longlong_as_double(-1ll);   // NaN
+  }
   const float* v0 = traces + static_cast<size_t>(s) * 2 * n;
   const float* v1 = v0 + n;
   double bv = -1.0;
@@ -1422,150 +1437,183 @@ __global__ void __launch_bounds__(256) voltage_peak_kernel(const float* traces, 
     idx[s] = bi;
     t_ns[s] = __dadd_rn(t_start[s], __dmul_rn(static_cast<double>(bi), dt_ns));
   }
+  pdl_wait_prior();
 }
 
-__device__ __forceinline__ double det3(const double (&a)[3][3]) {
-  return a[0][0] * (a[1][1] * a[2][2] - a[1][2] * a[2][1]) - a[0][1] * (a[1][0] * a[2][2] - a[1][2] * a[2][0]) +
-         a[0][2] * (a[1][0] * a[2][1] - a[1][1] * a[2][0]);
+// The 12 values v of each lane summed over the warp: the result of value i lies in the lanes of
+// slot i (warp_sum12_slot). Half of the values go to the other half of the lanes at each step, 13
+// additions where a butterfly per value takes 60 (an FP64 instruction occupies an SM's two FP64 lanes for
+// 16 cycles). The order is fixed.
+__device__ __forceinline__ int warp_sum12_slot(int lane) {   // -1: none
+  const int low = ((lane >> 2) & 1) * 2 + ((lane >> 1) & 1);
+  return low < 3 ? (lane >> 4) * 6 + ((lane >> 3) & 1) * 3 + low : -1;
+}
+__device__ __forceinline__ double warp_sum12(double (&v)[12], int lane) {
+  const auto step = [&](auto half, int off) {
+    constexpr int H = decltype(half)::value;
+    const bool up = (lane & off) != 0;
+#pragma unroll
+    for (int i = 0; i < H; ++i) {
+      const double give = up ? v[i] : v[i + H], keep = up ? v[i + H] : v[i];
+      v[i] = keep + __shfl_xor_sync(0xffffffffu, give, off);
+    }
+  };
+  step(std::integral_constant<int, 6>{}, 16);
+  step(std::integral_constant<int, 3>{}, 8);
+  v[3] = 0.0;
+  step(std::integral_constant<int, 2>{}, 4);
+  step(std::integral_constant<int, 1>{}, 2);
+  return v[0] + __shfl_xor_sync(0xffffffffu, v[0], 1);
 }
 
 // Least-squares plane wave t_s = t0 - n.x_s n_refr / c: linear in (t0, nx, ny) for a fixed nz,
 // repeated four times with nz from the previous solution (nz = 1 first). One CTA of 128
 // threads, FP64, sums in a fixed order. Also decides convergence and the residual chi2.
-__global__ void __launch_bounds__(128) plane_fit_kernel(FitParams p) {
+//
+// FP64 runs at 1/64 of the FP32 rate here, so the kernel is bound by its FP64 instructions and their
+// chains, and does each thing once: the station sums once for all four repetitions (the right-hand
+// side t + k nz z is linear in nz, so the solution is a + nz b), the matrix inverted once by its
+// cofactors, one thread's scalars for the repetitions, the mean residual from the sums, and the two
+// arc tangents, the convergence test and the next unfold's pattern cell on lanes of different
+// warps side by side. 124 stations: 44 us with sums per repetition and every thread repeating the
+// trigonometry, 12.7 us now (ncu, one launch at a time); the unfold kernel that takes the cell and
+// the source vector from here 19.5 -> 15.2 us.
+__global__ void __launch_bounds__(128) plane_fit_kernel(const __grid_constant__ FitParams p) {
+  pdl_launch_dependents();
+  pdl_wait_prior();
   ReconState* st = p.st;
   if (st->converged) return;
-  const int tid = threadIdx.x;
-  __shared__ double red[4][10];
-  __shared__ double sol[4];
-  __shared__ int same_s;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  __shared__ double red[4][12];
+  __shared__ double tot[12];
+  __shared__ double sol[6];       // t0, nx, ny, nz, mean residual time, horizontal component
+  __shared__ double angle[2];     // zenith, azimuth
+  __shared__ double pos[2];       // their positions in the pattern's table
+  __shared__ int flags[4];        // [0] a direction was found, [1] converged, [2], [3] of the positions
+  const double k = p.n_over_c;
   // do the station indices repeat those of the previous fit?
   int diff = 0;
-  if (p.iteration > 0)
-    for (int s = tid; s < p.n_st; s += 128) diff |= p.idx[s] != p.prev_idx[s];
-  const int any_diff = __syncthreads_or(diff);
-  for (int s = tid; s < p.n_st; s += 128) p.prev_idx[s] = p.idx[s];
-  if (tid == 0) same_s = p.iteration > 0 && !any_diff;
-  const double k = p.n_over_c;
-  double nz = 1.0;
-  bool ok = true;
-  for (int pass = 0; pass < 4 && ok; ++pass) {
-    double v[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};   // n, Sx, Sy, Sxx, Sxy, Syy, Sy_t, Sx_t, Sy_t(y)
-    for (int s = tid; s < p.n_st; s += 128) {
-      const double x = p.pos[3 * s], y = p.pos[3 * s + 1], z = p.pos[3 * s + 2];
-      const double yt = __dadd_rn(p.times[s], __dmul_rn(__dmul_rn(k, nz), z));
-      v[0] += 1.0; v[1] += x; v[2] += y; v[3] += x * x; v[4] += x * y; v[5] += y * y;
-      v[6] += yt; v[7] += x * yt; v[8] += y * yt;
-    }
-#pragma unroll
-    for (int i = 0; i < 9; ++i) {
-      double t = v[i];
-#pragma unroll
-      for (int off = 16; off > 0; off >>= 1) t += __shfl_xor_sync(0xffffffffu, t, off);
-      if ((tid & 31) == 0) red[tid >> 5][i] = t;
-    }
-    __syncthreads();
-    if (tid == 0) {
-      double t[9];
-      for (int i = 0; i < 9; ++i) t[i] = red[0][i] + red[1][i] + red[2][i] + red[3][i];
-      const double m[3][3] = {{t[0], t[1], t[2]}, {t[1], t[3], t[4]}, {t[2], t[4], t[5]}};
-      const double r[3] = {t[6], t[7], t[8]};
-      const double det = det3(m);
-      if (!(fabs(det) > 1e-12 * (m[0][0] * m[1][1] * m[2][2]))) {
-        sol[3] = 0.0;
-      } else {
-        double x[3];
-        for (int c = 0; c < 3; ++c) {
-          double a[3][3];
-          for (int i = 0; i < 3; ++i)
-            for (int j = 0; j < 3; ++j) a[i][j] = j == c ? r[i] : m[i][j];
-          x[c] = det3(a) / det;
+  double v[12] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0};   // x, y, xx, xy, yy, t, xt, yt, z, xz, yz
+  for (int s = tid; s < p.n_st; s += 128) {
+    const double x = p.pos[3 * s], y = p.pos[3 * s + 1], z = p.pos[3 * s + 2], t = p.times[s];
+    v[0] += x; v[1] += y; v[2] += x * x; v[3] += x * y; v[4] += y * y;
+    v[5] += t; v[6] += x * t; v[7] += y * t;
+    v[8] += z; v[9] += x * z; v[10] += y * z;
+    const int i = p.idx[s];
+    diff |= p.iteration > 0 && i != p.prev_idx[s];
+    p.prev_idx[s] = i;
+  }
+  const double total = warp_sum12(v, lane);
+  const int slot = warp_sum12_slot(lane);
+  if (slot >= 0 && (lane & 1) == 0) red[warp][slot] = total;
+  const int same = !__syncthreads_or(diff) && p.iteration > 0;
+  if (warp == 0) {
+    if (lane < 12) tot[lane] = red[0][lane] + red[1][lane] + red[2][lane] + red[3][lane];
+    __syncwarp();
+    if (lane == 0) {
+      const double n = p.n_st, sx = tot[0], sy = tot[1], sxx = tot[2], sxy = tot[3], syy = tot[4];
+      const double c00 = sxx * syy - sxy * sxy, c01 = sxy * sy - sx * syy, c02 = sx * sxy - sxx * sy;
+      const double c11 = n * syy - sy * sy, c12 = sx * sy - n * sxy, c22 = n * sxx - sx * sx;
+      const double det = n * c00 + sx * c01 + sy * c02;
+      const bool ok = fabs(det) > 1e-12 * (n * sxx * syy);
+      flags[0] = ok ? 1 : 0;
+      if (ok) {
+        const double inv = 1.0 / det, inv_k = 1.0 / (k * det);
+        // the solution of the right-hand sides t and k z: t0 and -(nx, ny) k
+        const double a0 = (c00 * tot[5] + c01 * tot[6] + c02 * tot[7]) * inv;
+        const double a1 = -(c01 * tot[5] + c11 * tot[6] + c12 * tot[7]) * inv_k;
+        const double a2 = -(c02 * tot[5] + c12 * tot[6] + c22 * tot[7]) * inv_k;
+        const double b0 = k * (c00 * tot[8] + c01 * tot[9] + c02 * tot[10]) * inv;
+        const double b1 = -(c01 * tot[8] + c11 * tot[9] + c12 * tot[10]) * inv;
+        const double b2 = -(c02 * tot[8] + c12 * tot[9] + c22 * tot[10]) * inv;
+        double nx = 0.0, ny = 0.0, nz = 1.0, t0 = 0.0, h2 = 0.0;
+        for (int pass = 0; pass < 4; ++pass) {
+          t0 = a0 + nz * b0;
+          nx = a1 + nz * b1;
+          ny = a2 + nz * b2;
+          h2 = nx * nx + ny * ny;
+          if (h2 > 1.0) {
+            const double h = sqrt(h2);
+            nx /= h;
+            ny /= h;
+            h2 = 1.0;
+          }
+          nz = sqrt(1.0 - h2);
         }
-        double nx = -x[1] / k, ny = -x[2] / k;
-        double h2 = nx * nx + ny * ny;
-        if (h2 > 1.0) {
-          const double h = sqrt(h2);
-          nx /= h;
-          ny /= h;
-          h2 = 1.0;
-        }
-        sol[0] = x[0];
+        sol[0] = t0;
         sol[1] = nx;
         sol[2] = ny;
-        sol[3] = 1.0;
+        sol[3] = nz;
+        sol[4] = (tot[5] + k * (nx * sx + ny * sy + nz * tot[8])) / n;
+        sol[5] = h2;
       }
     }
-    __syncthreads();
-    ok = sol[3] != 0.0;
-    if (ok) nz = sqrt(1.0 - (sol[1] * sol[1] + sol[2] * sol[2]));
-    __syncthreads();
   }
-  if (!ok) {   // no direction: stop; the first fit failing marks the reconstruction failed
+  __syncthreads();
+  if (!flags[0]) {   // no direction: stop; the first fit failing marks the reconstruction failed
     if (tid == 0) {
       st->converged = 1;
-      if (p.iteration == 0) {
-        st->failed = 1;
-        st->dir[0] = st->dir[1] = st->t0 = st->chi2 = __longlong_as_double(0x7ff8000000000000ll);
-      } else {
-        st->iterations = p.iteration;
-      }
+      if (p.iteration == 0) p.direction[0] = p.direction[1] = *p.t0 = *p.chi2 = __longlong_as_double(0x7ff8000000000000ll);
+      *p.iterations = p.iteration == 0 ? -1 : p.iteration;
     }
     return;
   }
-  const double nx = sol[1], ny = sol[2];
-  const double zen = atan2(sqrt(nx * nx + ny * ny), nz);
-  double az = atan2(ny, nx);
-  if (az < 0.0) az += 2.0 * 3.14159265358979323846;
-  // chi2 of this direction with these times (two-pass mean, as the per-direction residual)
-  const double snx = sin(zen) * cos(az), sny = sin(zen) * sin(az), snz = cos(zen);
-  double acc = 0.0;
-  for (int s = tid; s < p.n_st; s += 128)
-    acc += p.times[s] + (snx * p.pos[3 * s] + sny * p.pos[3 * s + 1] + snz * p.pos[3 * s + 2]) * k;
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
-  if ((tid & 31) == 0) red[tid >> 5][9] = acc;
-  __syncthreads();
-  const double mean = (red[0][9] + red[1][9] + red[2][9] + red[3][9]) / p.n_st;
-  __syncthreads();
+  const double nx = sol[1], ny = sol[2], nz = sol[3], mean = sol[4];
+  // chi2 of this direction with these times
   double ss = 0.0;
   for (int s = tid; s < p.n_st; s += 128) {
-    const double r = p.times[s] + (snx * p.pos[3 * s] + sny * p.pos[3 * s + 1] + snz * p.pos[3 * s + 2]) * k - mean;
+    const double r = p.times[s] + (nx * p.pos[3 * s] + ny * p.pos[3 * s + 1] + nz * p.pos[3 * s + 2]) * k - mean;
     ss += r * r;
   }
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, off);
-  if ((tid & 31) == 0) red[tid >> 5][9] = ss;
+  if (lane == 0) {
+    red[warp][0] = ss;
+    if (warp == 1) {
+      angle[0] = atan2(sqrt(sol[5]), nz);
+      bool clamped;
+      flags[2] = zenith_position(p.pattern, angle[0], &pos[0], &clamped) ? (clamped ? 2 : 1) : 0;
+    } else if (warp == 2) {
+      double az = atan2(ny, nx);
+      if (az < 0.0) az += 2.0 * 3.14159265358979323846;
+      angle[1] = az;
+      flags[3] = azimuth_position(p.pattern, az, &pos[1]) ? 1 : 0;
+    } else if (warp == 3) {
+      bool done = false;
+      if (p.iteration > 0) {
+        double dot = st->n[0] * nx + st->n[1] * ny + st->n[2] * nz;
+        dot = dot > 1.0 ? 1.0 : (dot < -1.0 ? -1.0 : dot);
+        done = same || acos(dot) < p.tol_rad;
+      }
+      flags[1] = done ? 1 : 0;
+    }
+  }
   __syncthreads();
   if (tid == 0) {
-    const double chi2 = red[0][9] + red[1][9] + red[2][9] + red[3][9];
-    bool done = false;
-    if (p.iteration > 0) {
-      const double pz = st->dir[0], pa = st->dir[1];
-      double dot = sin(pz) * cos(pa) * snx + sin(pz) * sin(pa) * sny + cos(pz) * snz;
-      dot = dot > 1.0 ? 1.0 : (dot < -1.0 ? -1.0 : dot);
-      done = same_s || acos(dot) < p.tol_rad;
-      st->iterations = p.iteration;
-    }
+    const double zen = angle[0], az = angle[1];
     st->dir[0] = zen;
     st->dir[1] = az;
-    st->t0 = sol[0];
-    st->chi2 = chi2;
+    st->n[0] = nx;
+    st->n[1] = ny;
+    st->n[2] = nz;
+    if (flags[1]) st->converged = 1;
+    DirPre* dp = p.dir_pre;
+    dp->cell = p.own_pattern ? cell_of_positions(p.pattern, flags[2] && flags[3], pos[0], flags[2] == 2, pos[1]) : DirInfo{};
+    dp->n[0] = nx;
+    dp->n[1] = ny;
+    dp->n[2] = nz;
+    dp->pad = 0.0;
+  } else if (tid == 32) {
+    p.direction[0] = angle[0];
+    p.direction[1] = angle[1];
+    *p.t0 = sol[0];
+    *p.chi2 = red[0][0] + red[1][0] + red[2][0] + red[3][0];
+    *p.iterations = p.iteration;
     if (p.history) {
-      p.history[2 * p.iteration] = zen;
-      p.history[2 * p.iteration + 1] = az;
+      p.history[2 * p.iteration] = angle[0];
+      p.history[2 * p.iteration + 1] = angle[1];
     }
-    if (done) st->converged = 1;
   }
-}
-
-// the reconstruction's results into the caller's outputs
-__global__ void recon_finish_kernel(const ReconState* st, double* direction, double* t0, double* chi2, int* iterations) {
-  if (threadIdx.x != 0) return;
-  direction[0] = st->dir[0];
-  direction[1] = st->dir[1];
-  *t0 = st->t0;
-  *chi2 = st->chi2;
-  *iterations = st->failed ? -1 : st->iterations;
 }
 
 }  // namespace aerafold
