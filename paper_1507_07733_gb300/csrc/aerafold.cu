@@ -475,12 +475,28 @@ EventDesc make_desc(const PathBuffers& b, const ar_pattern_desc& pd, const float
   return d;
 }
 
-// One event: the station kernel (one CTA per station), then the persistent unfold kernel.
-// The station kernel is launched in plain stream order: launched early behind the previous
-// call's unfold kernel it would hold SM slots that kernel's successor needs (back to back,
-// calls took 0.124 instead of 0.095 ms on the scan). The unfold kernel is launched with
-// programmatic dependent launch, so its CTAs start while the station kernel runs and fetch
-// their first corner slabs before they wait for the spectra.
+// The station kernel (one CTA per station) of an event, launched early behind whatever is before
+// it in the stream and waiting for it before it touches anything: its CTAs take their places as the
+// previous call's leave, which saves the launch latency (calls back to back at 2048 samples: 10 x 1
+// pairs 14.4 -> 12.2 us, 124 x 8 24.2 -> 22.4, 124 x 64 78.0 -> 75.8). Where the unfold kernel has
+// two CTAs per SM (4096 samples), one pair for each, and the station kernel's 72 KB beside one of
+// them leaves too few places, its CTAs crowd onto the SMs that free up first and hold up the
+// unfold kernel (124 x 2 pairs 23.3 -> 25.0 us, 100 x 3 22.9 -> 24.8; with room 76 x 3 20.5 -> 18.5, with
+// several pairs per CTA 124 x 5 29.4 -> 27.7): plain stream order there.
+template <int N_>
+cudaError_t launch_station(PathParams pp, long long pairs, int grid_cap, cudaStream_t stream) {
+  const int S = pp.ev0.n_st;
+  if (Layout<N_>::MIN_CTAS == 2 && pairs <= grid_cap && pairs + S > grid_cap) {
+    station_spectrum_kernel<N_><<<S, SpectrumSmem<N_>::BLOCK, SpectrumSmem<N_>::TOTAL, stream>>>(pp);
+    return cudaGetLastError();
+  }
+  pp.wait_first = 1;
+  return launch_pdl(station_spectrum_kernel<N_>, S, SpectrumSmem<N_>::BLOCK, SpectrumSmem<N_>::TOTAL, stream, pp);
+}
+
+// One event: the station kernel, then the persistent unfold kernel, launched with programmatic
+// dependent launch, so its CTAs start while the station kernel runs and build their first inverse
+// before they wait for the spectra.
 template <int N_>
 cudaError_t launch_path(unsigned* err, const EventDesc& desc, int grid_cap, cudaStream_t stream,
                         cudaEvent_t* evs /* 3 events or null */, int test_wait = 0) {
@@ -493,10 +509,9 @@ cudaError_t launch_path(unsigned* err, const EventDesc& desc, int grid_cap, cuda
   pp.ev0 = desc;
   cudaError_t e;
   if (evs && (e = cudaEventRecord(evs[0], stream)) != cudaSuccess) return e;
-  station_spectrum_kernel<N_><<<desc.n_st, SpectrumSmem<N_>::BLOCK, SpectrumSmem<N_>::TOTAL, stream>>>(pp);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  if (evs && (e = cudaEventRecord(evs[1], stream)) != cudaSuccess) return e;
   const long long pairs = static_cast<long long>(desc.n_st) * desc.n_dir;
+  if ((e = launch_station<N_>(pp, pairs, grid_cap, stream)) != cudaSuccess) return e;
+  if (evs && (e = cudaEventRecord(evs[1], stream)) != cudaSuccess) return e;
   const long long grid = std::min<long long>(grid_cap, pairs);
   const size_t smem = UnfoldSmem<N_>::total(pp.ev0.n_f_layout, pp.ev0.slab_direct != 0);
   if ((e = desc.snr ? launch_pdl(unfold_kernel<N_, true>, static_cast<int>(grid), L::T, smem, stream, pp)
@@ -739,8 +754,7 @@ cudaError_t launch_recon(ar_ctx* ctx, const ar_event* ev, int max_iter, double t
   PathParams sp = pp;
   sp.skip = nullptr;
   sp.ev0.dir_pre = nullptr;
-  station_spectrum_kernel<N_><<<S, SpectrumSmem<N_>::BLOCK, SpectrumSmem<N_>::TOTAL, stream>>>(sp);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  if ((e = launch_station<N_>(sp, S, rs.kc->grid, stream)) != cudaSuccess) return e;
   // every kernel from here on is launched early behind the previous one and waits for it
   const int n_history = 2 * (max_iter + 1);
   if ((e = launch_pdl(voltage_peak_kernel, S, 256, 0, stream, ev->traces, ev->t_start_ns, static_cast<int>(ev->n_samples),

@@ -241,6 +241,7 @@ struct PathParams {
   unsigned* err;              // device error word
   const int* skip;            // if not null and *skip != 0 the kernel does nothing (a loop has converged)
   int wait_prior;             // wait for the previous kernel in the stream (its results are needed)
+  int wait_first;             // (station kernel) wait for it before anything else: launched early behind any kernel
   // Test of the bounded-wait error path (ar_set_test_fault): nonzero makes every corner-slab
   // mbarrier expect 16 bytes more than its four bulk copies deliver, and its waits give up
   // after 1 ms, so the waits run out, the error word gets kErrTmaTimeout and the CTAs return.
@@ -374,6 +375,7 @@ __global__ void __launch_bounds__(SpectrumSmem<N_>::BLOCK) station_spectrum_kern
   float2* x1 = reinterpret_cast<float2*>(smem_raw + SM::X1);
   float2* tw = reinterpret_cast<float2*>(smem_raw + SM::TW);
   const int tid = threadIdx.x;
+  if (prm.wait_first) pdl_wait_prior();
   pdl_launch_dependents();
   // threads [0, T) transform (their barriers are named barrier 1); the last warp forms the
   // per-direction entries meanwhile (directions s, s + S, ... of the event for station s)
