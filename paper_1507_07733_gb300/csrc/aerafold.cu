@@ -1096,16 +1096,12 @@ cudaError_t launch_gemm(ar_ctx* ctx, __nv_bfloat16* const (&a)[3], size_t m_pad,
   gp.groups = groups;
   // persistent: one CTA per SM (the kernel's shared memory allows one), items strided
   const int items = tiles * groups;
-  if (wide)
-    tc::split_gemm_kernel<256><<<std::min(items, ctx->num_sms), tc::kGemmThreads, tc::kGemmSmem, stream>>>(gp);
-  else
-    tc::split_gemm_kernel<128><<<std::min(items, ctx->num_sms), tc::kGemmThreads, tc::kGemmSmem, stream>>>(gp);
-  cudaError_t e = cudaGetLastError();
+  cudaError_t e = launch_pdl(wide ? tc::split_gemm_kernel<256> : tc::split_gemm_kernel<128>,
+                             std::min(items, ctx->num_sms), tc::kGemmThreads, tc::kGemmSmem, stream, gp);
   if (e != cudaSuccess || groups == 1) return e;
   const size_t n4 = gp.d_group / 4;
-  tc::tc_reduce_kernel<<<2 * ctx->num_sms, 256, 0, stream>>>(reinterpret_cast<const float4*>(part),
-                                                              reinterpret_cast<float4*>(d), n4, n4, groups);
-  return cudaGetLastError();
+  return launch_pdl(tc::tc_reduce_kernel, 2 * ctx->num_sms, 256, 0, stream, reinterpret_cast<const float4*>(part),
+                    reinterpret_cast<float4*>(d), n4, n4, groups);
 }
 
 template <int N_>
@@ -1122,8 +1118,13 @@ cudaError_t launch_tc(ar_ctx* ctx, const EventDesc& ev, int terms, size_t rows_f
   const bool prof = ctx->profiling;
   cudaError_t e;
   if (prof && (e = cudaEventRecord(ctx->ev[0], stream)) != cudaSuccess) return e;
-  tc::tc_forward_pre_kernel<N_><<<2 * S, tc::kSub, 0, stream>>>(ev, fimg);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  // The kernels are launched early behind the one before them and wait for it, all but the solve and
+  // the post-pass: their many CTAs, started one by one as the GEMM's or the reduction's leave, fill
+  // the SMs unevenly (43 x 29 pairs at 4096 samples, x6: all in stream order 129.6 us, all early 147, these
+  // two in stream order 122.5; 124 x 64 at 2048, x3: 238, 253, 230; 10 x 1 at 4096: 51, 41, 37).
+  if ((e = launch_pdl(tc::tc_forward_pre_kernel<N_>, 2 * S + (D + tc::kTcDirsPerCta - 1) / tc::kTcDirsPerCta, tc::kSub,
+                      0, stream, ev, fimg)) != cudaSuccess)
+    return e;
   if ((e = launch_gemm(ctx, w.fa, rows_f, 0, terms, w.xf, w.part, stream)) != cudaSuccess) return e;
   // per-bin inverses [2][N/4] float4, then the node scratch [n_f][8] float2
   const size_t solve_smem = 2 * sizeof(float4) * (N_ / 4) + sizeof(float2) * 8 * static_cast<size_t>(ev.n_f_layout);
@@ -1149,8 +1150,7 @@ cudaError_t launch_tc(ar_ctx* ctx, const EventDesc& ev, int terms, size_t rows_f
     tc::tc_inverse_post_kernel<N_><<<np, tc::kSub, 0, stream>>>(ev, reinterpret_cast<const float2*>(w.yi), p0);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
-  tc::tc_residual_kernel<<<D, 128, 0, stream>>>(ev);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  if ((e = launch_pdl(tc::tc_residual_kernel, D, 128, 0, stream, ev)) != cudaSuccess) return e;
   if (prof && (e = cudaEventRecord(ctx->ev[3], stream)) != cudaSuccess) return e;
   return cudaSuccess;
 }
@@ -1197,7 +1197,7 @@ ar_status ar_unfold_tc(ar_ctx* ctx, const ar_event* ev, const ar_outputs* out, i
     ctx->tc_ws_bytes = need;
   }
   const PatternDev& pat = ctx->patterns[ev->pattern_id];
-  PathBuffers b{ctx->spec, ctx->dir_done, ctx->d_err, rs.lt->t1, rs.lt->wn, rs.binf};
+  PathBuffers b{ctx->spec, ctx->dir_done, ctx->d_err, rs.lt->t1, rs.lt->wn, rs.binf, ctx->dir_pre};
   EventDesc desc = make_desc(b, pat.desc, pat.table, ev, out, rs.k_lo);
   if ((st = attach_patterns(ctx, ev, rs.k_lo, &desc)) != AR_OK) return st;
   cudaStream_t s = static_cast<cudaStream_t>(stream);

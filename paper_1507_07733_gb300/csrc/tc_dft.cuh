@@ -208,6 +208,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) split_gemm_kernel(const __gri
   uint64_t* done = bars + 10;     // every MMA complete
   uint32_t* taddr_s = reinterpret_cast<uint32_t*>(bars + 11);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  pdl_launch_dependents();
   const int items = p.m_tiles * p.n_tiles * p.groups;
   // Persistent: this CTA takes items blockIdx.x, blockIdx.x + gridDim.x, ...; their chunks
   // form one stream (chunk i of the stream is chunk i % cpg of item i / cpg), so one item's
@@ -244,6 +245,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) split_gemm_kernel(const __gri
   tc_fence_after();
   const uint32_t t_sum = *taddr_s;
   bool ok = true;
+  pdl_wait_prior();   // A comes from the previous kernel, and D may still be read by an earlier one
 
   if (warp == 4) {
     // ---- producer: bulk copies of each chunk's A and B blocks into a free stage ----
@@ -359,6 +361,8 @@ __global__ void __launch_bounds__(kGemmThreads, 1) split_gemm_kernel(const __gri
 // Sum of the split-K groups' partial results, in group order (each group already folded its
 // chunks in order): out[i] = ((part[0][i] + part[1][i]) + ...).
 __global__ void tc_reduce_kernel(const float4* part, float4* out, size_t n4, size_t group4, int groups) {
+  pdl_launch_dependents();
+  pdl_wait_prior();
   for (size_t i = blockIdx.x * static_cast<size_t>(blockDim.x) + threadIdx.x; i < n4;
        i += static_cast<size_t>(gridDim.x) * blockDim.x) {
     float4 a = part[i];
@@ -372,7 +376,10 @@ __global__ void tc_reduce_kernel(const float4* part, float4* out, size_t n4, siz
 
 // ---- forward: phase rotation, A-point DFT over the sub-block phase, twiddle ----------------
 // One CTA per (station, channel), thread n2; writes W[j1][n2] as GEMM row ((s * 2 + c) * A + j1),
-// complex column n2, into the BF16 planes of the forward GEMM's A image.
+// complex column n2, into the BF16 planes of the forward GEMM's A image. The CTAs behind those form the
+// directions' entries (kTcDirsPerCta each: cells and source vectors, 3 us of FP64 chains that every
+// solve and residual CTA repeated).
+constexpr int kTcDirsPerCta = 8 * (kSub / 32);
 struct SplitImage {
   __nv_bfloat16* plane[3];
   int planes;
@@ -383,6 +390,13 @@ __global__ void __launch_bounds__(kSub) tc_forward_pre_kernel(const __grid_const
                                                               const __grid_constant__ SplitImage img) {
   constexpr int N = N_, A = N / kSub;
   const int sc = blockIdx.x, n2 = threadIdx.x;
+  pdl_wait_prior();   // the caller's inputs and the previous call's buffers
+  pdl_launch_dependents();
+  if (sc >= 2 * ev.n_st) {
+    const int d = (sc - 2 * ev.n_st) * kTcDirsPerCta + (n2 >> 2);   // eight directions a warp, four lanes each
+    precompute_direction(ev, d, n2 & 3, d < ev.n_dir);
+    return;
+  }
   const float* x = ev.traces + static_cast<size_t>(sc) * N;
   float2 y[A];
 #pragma unroll
@@ -427,6 +441,7 @@ __global__ void __launch_bounds__(kSolveThreads) tc_solve_kernel(const __grid_co
   int cur_d = -1, cur_p = -3;
   DirInfo di;
   bool key_sing = false;
+  pdl_launch_dependents();
   for (int k = 0; k < pairs_per_cta; ++k) {
     const int lp = blockIdx.x * pairs_per_cta + k;   // pair within the chunk
     if (lp >= n_pairs) break;
@@ -434,10 +449,10 @@ __global__ void __launch_bounds__(kSolveThreads) tc_solve_kernel(const __grid_co
     const int d = static_cast<int>(pair / S), s = static_cast<int>(pair % S);
     const int p = station_pattern(ev, s);
     if (d != cur_d || p != cur_p) {
-      // new direction or pattern: the cell (FP64) by one thread (FP64 is a small fraction of
-      // the FP32 rate), then the per-bin inverse
+      // new direction or pattern: the cell (the event's own pattern's from the direction's entry,
+      // a station's own formed by one thread), then the per-bin inverse
       __syncthreads();   // the previous pair's reads of hinv are done
-      if (tid == 0) s_di = pair_cell(ev, d, p, nullptr);
+      if (tid == 0) s_di = p == -1 ? load_cell(ev.dir_pre + d) : pair_cell(ev, d, p, nullptr);
       __syncthreads();
       di = s_di;
       key_sing = build_inverse<N_, T>(ev, p, di, nullptr, true, hn, hinv);
@@ -475,6 +490,7 @@ __global__ void __launch_bounds__(kSub) tc_inverse_post_kernel(const __grid_cons
   const int lp = blockIdx.x, n2 = threadIdx.x;
   const long long pair = pair0 + lp;
   const int s = static_cast<int>(pair % ev.n_st);
+  pdl_launch_dependents();
   float pw[A];
 #pragma unroll
   for (int i = 0; i < A; ++i) pw[i] = 0.f;
@@ -540,8 +556,12 @@ __global__ void __launch_bounds__(kSub) tc_inverse_post_kernel(const __grid_cons
 }
 
 // ---- per direction: the FP64 plane-wave timing residual ------------------------------------
+// A kernel of its own: with a completion counter in the post-pass, whose CTA per pair lives only a few
+// microseconds, the release of every pair took that kernel from 29.5 to 43 us (1247 pairs at 4096).
 __global__ void __launch_bounds__(128) tc_residual_kernel(const __grid_constant__ EventDesc ev) {
   __shared__ double red[128 / 32];
+  pdl_launch_dependents();
+  pdl_wait_prior();
   direction_residual<128>(ev, blockIdx.x, red);
 }
 
