@@ -77,11 +77,13 @@ struct Layout : Shape<N_> {
   static constexpr int A_F2 = 8 * PLN;                // A: [pol][r][row][mb]; E aliases it
   static_assert(SPLIT == 1 || SPLIT == 2, "layout");
   static_assert(A_F2 >= 2 * S::M, "E must fit in A");
-  // with SPLIT == 2, the |Y|^2 exchange between the two polarisations' threads, P x 4Q
-  // floats, also reuses A once pass 2 has read it
-  static_assert(2 * A_F2 >= S::P * 4 * S::Q, "the exchange must fit in A");
-  // outputs staged behind E: 16M bytes of E (or the exchange), then 3N floats
-  static_assert(sizeof(float2) * A_F2 >= 16 * S::M + 12 * S::N, "the output staging must fit in A");
+  // Outputs staged behind E (16M bytes): e_theta, e_phi, the envelope, N floats each. With SPLIT == 2 a
+  // warp's two half-warps write 16 samples of one polarisation each, or of one half of the envelope,
+  // a multiple of 32 apart: e_phi and the envelope's second half lie 16 floats further, in other banks.
+  static constexpr int SKEW = SPLIT == 2 ? 16 : 0;
+  static constexpr int STAGE_P = S::N + SKEW;                  // e_phi
+  static constexpr int STAGE_V = 2 * S::N + 2 * SKEW;          // the envelope
+  static_assert(sizeof(float2) * A_F2 >= 16 * S::M + 4 * (STAGE_V + S::N + SKEW), "the output staging must fit in A");
   static_assert(T % 32 == 0 && S::M % T == 0, "layout");
 };
 
@@ -667,9 +669,10 @@ struct UnfoldSmem {
 
 // Sub-sample offset of the envelope maximum at sample k: the vertex of the parabola through
 // (k-1, k, k+1), in FP64; 0 at the trace ends or without a strict maximum, clamped to +-1/2.
-__device__ __forceinline__ double peak_offset(const float* env, int n, int k) {
+template <typename F>
+__device__ __forceinline__ double peak_offset(F env, int n, int k) {
   if (k <= 0 || k >= n - 1) return 0.0;
-  const double a = env[k - 1], b = env[k], c = env[k + 1];
+  const double a = env(k - 1), b = env(k), c = env(k + 1);
   const double second = __dadd_rn(__dsub_rn(a, __dmul_rn(2.0, b)), c);
   if (!(second < 0.0)) return 0.0;
   const double delta = __ddiv_rn(__dmul_rn(0.5, __dsub_rn(a, c)), second);
@@ -679,22 +682,23 @@ __device__ __forceinline__ double peak_offset(const float* env, int n, int k) {
 // Pulse SNR of a pair (a variant; the paper defines no noise estimate): (peak / noise)^2 at
 // the envelope maximum k, noise^2 the mean of env^2 over the samples more than n/16 from k;
 // 0 when there are none or their mean is 0. Whole CTA over the envelope in shared memory:
-// thread t sums samples t, t + T, ..., the warps combine in a fixed tree and thread 0 adds the
-// warps in order; the result is thread 0's. red holds T/32 floats.
-template <int T>
-__device__ __forceinline__ float pair_snr(const float* env, int n, int k, float peak, float* red) {
+// thread t sums samples t, t + T, ..., the warps combine in a fixed tree and thread LEAD adds the
+// warps in order; the result is that thread's. red holds T/32 floats.
+template <int T, int LEAD, typename F>
+__device__ __forceinline__ float pair_snr(F env, int n, int k, float peak, float* red) {
   const int w = n / 16;
   float acc = 0.f;
   for (int i = threadIdx.x; i < n; i += T) {
     const int dd = i > k ? i - k : k - i;
-    if (dd > w) acc = fmaf(env[i], env[i], acc);
+    const float v = env(i);
+    if (dd > w) acc = fmaf(v, v, acc);
   }
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
   __syncthreads();
   float snr = 0.f;
-  if (threadIdx.x == 0) {
+  if (threadIdx.x == LEAD) {
     float ss = red[0];
 #pragma unroll
     for (int i = 1; i < T / 32; ++i) ss += red[i];
@@ -1024,6 +1028,13 @@ __global__ void __launch_bounds__(Layout<N_>::T, Layout<N_>::MIN_CTAS) unfold_ke
   float2* slab = reinterpret_cast<float2*>(smem_raw + SM::SLAB);
 
   const int tid = threadIdx.x;
+  // What one thread does at a pair's end holds up the others at the next barrier, so three warps share
+  // it: threads 0 and 32 issue the staged outputs' copies, thread kPeakLead combines the warps'
+  // peaks and stores the results (one thread for all: scan of 67 x 51 pairs at 4096 samples 82.5 us,
+  // two 80.0; 101 x 97 at 1024 56.5 and 54.0).
+  constexpr int kPeakLead = 64;
+  static_assert(T > kPeakLead, "three warps");
+  const bool copies_out = tid == 0 || tid == 32;
 
   // the launch's events and the contiguous chunk of its flattened pair space for this CTA
   const EventDesc* evs = prm.batch ? batch_events(prm.batch) : &prm.ev0;
@@ -1106,8 +1117,8 @@ __global__ void __launch_bounds__(Layout<N_>::T, Layout<N_>::MIN_CTAS) unfold_ke
           if (tid == 0) {
             atomicOr(prm.err, kErrTmaTimeout);
             mbar_wait_bounded(bar, phase, limit);
-            tma_bulk_wait_all();
           }
+          if (copies_out) tma_bulk_wait_all();
           __syncthreads();
           return;
         }
@@ -1124,7 +1135,7 @@ __global__ void __launch_bounds__(Layout<N_>::T, Layout<N_>::MIN_CTAS) unfold_ke
       // the inverse of every bin, shared by the key's stations. The node scratch overlays A: the
       // previous pair's staged outputs must have left it.
       di = *sdir;
-      if (tid == 0) tma_bulk_wait_read();
+      if (copies_out) tma_bulk_wait_read();
       __syncthreads();
       key_sing = build_inverse<N_>(ev, p, di, slab, ev.slab_direct != 0, hn, hinv, prm.err);
       run = (wants & kWalk) ? 0 : min(S - 1 - k, n_pairs - 1 - q);
@@ -1194,7 +1205,7 @@ __global__ void __launch_bounds__(Layout<N_>::T, Layout<N_>::MIN_CTAS) unfold_ke
       float2 x[Q];
       const float2* Ep = E + pol * M;
       pass1_task<N_>(Ep, ja, r, ev.k_lo, ev.t1, x);
-      if (tid == 0) tma_bulk_wait_read();   // the previous pair's staged outputs have left A
+      if (copies_out) tma_bulk_wait_read();   // the previous pair's staged outputs have left A
       __syncthreads();   // every E read done: A may overwrite it
       const int row = (ev.k_lo + ja) % P;
       float2* dst = A + (pol * 4 + r) * PLN + row * LDA;
@@ -1203,9 +1214,8 @@ __global__ void __launch_bounds__(Layout<N_>::T, Layout<N_>::MIN_CTAS) unfold_ke
     __syncthreads();
 
     // ---- pass 2: P-point DFTs, E-field, envelope, peak ----
-    // Outputs are staged in shared memory behind E (bytes [16M, 64M) of A: e_theta, e_phi,
-    // envelope, N floats each) and written by two bulk copies; with SPLIT == 2 the |Y|^2
-    // exchange uses the first 16M bytes (where E was).
+    // Outputs are staged in shared memory behind E (from byte 16M of A: e_theta, e_phi, envelope,
+    // see Layout) and written by bulk copies.
     const size_t pair = static_cast<size_t>(d) * S + s;
     // (debug build) the pair lies in the event's outputs; otherwise none of its outputs is written
     const bool pair_ok = in_bounds(e < n_events && d >= 0 && d < ev.n_dir && s >= 0 && s < S, prm.err);
@@ -1253,69 +1263,67 @@ __global__ void __launch_bounds__(Layout<N_>::T, Layout<N_>::MIN_CTAS) unfold_ke
           stage[n] = y0[ma].x;
           stage[N + n] = y1[ma].x;
         }
-        if (stage_env) stage[2 * N + n] = v;
+        if (stage_env) stage[L::STAGE_V + n] = v;
         if (v > bv) { bv = v; bi = n; }
       });
     } else {
       constexpr int TQ = 4 * Q;
-      const int pol = tid / TQ;             // warp-uniform
-      const int tq = tid % TQ;
+      const int pol = (tid >> 4) & 1;       // a half-warp each, for the same 16 (r, mb)
+      const int tq = (tid >> 5) * 16 + (tid & 15);
       const int r = tq & 3, mb = tq >> 2;
       float2 y[P];
       const float2* src = A + (pol * 4 + r) * PLN + mb;
       static_for<0, P>([&](auto i) { y[i] = src[i * LDA]; });
-      __syncthreads();   // every A read done: the exchange and the staging area may overwrite it
+      __syncthreads();   // every A read done: the staging area may overwrite it
       dft<P, +1>(y);
       float pw[P];
       static_for<0, P>([&](auto ma) {
         pw[ma] = cabs2(y[ma]);
-        if (traces) stage[pol * N + tq + TQ * ma] = y[ma].x;
+        if (traces) stage[pol * L::STAGE_P + tq + TQ * ma] = y[ma].x;
       });
-      // the theta threads publish the powers of samples ma in [P/2, P), the phi threads those
-      // of [0, P/2); each side then forms the envelope of the half it keeps ([P][TQ] floats)
-      float* xch = reinterpret_cast<float*>(A);
-      if (pol == 0) {
-        static_for<P / 2, P>([&](auto ma) { xch[ma * TQ + tq] = pw[ma]; });
-      } else {
-        static_for<0, P / 2>([&](auto ma) { xch[ma * TQ + tq] = pw[ma]; });
-      }
-      __syncthreads();
-      if (pol == 0) {
-        static_for<0, P / 2>([&](auto ma) {
-          const float v = sqrt_approx(pw[ma] + xch[ma * TQ + tq]);
-          if (stage_env) stage[2 * N + tq + TQ * ma] = v;
-          if (v > bv) { bv = v; bi = tq + TQ * ma; }
-        });
-      } else {
-        static_for<P / 2, P>([&](auto ma) {
-          const float v = sqrt_approx(pw[ma] + xch[ma * TQ + tq]);
-          if (stage_env) stage[2 * N + tq + TQ * ma] = v;
-          if (v > bv) { bv = v; bi = tq + TQ * ma; }
-        });
-      }
+      // the theta half forms the envelope of samples ma in [0, P/2), the phi half of [P/2, P), each
+      // with the other's power of the same sample (a shuffle; through shared memory it took two
+      // accesses and a barrier)
+      static_for<0, P / 2>([&](auto ma) {
+        constexpr int LO = decltype(ma)::value, HI = LO + P / 2;
+        const float other = __shfl_xor_sync(0xffffffffu, pol ? pw[LO] : pw[HI], 16);
+        const float v = sqrt_approx((pol ? pw[HI] : pw[LO]) + other);
+        const int n = tq + TQ * LO + pol * (N / 2);
+        if (stage_env) stage[L::STAGE_V + n + pol * L::SKEW] = v;
+        if (v > bv) { bv = v; bi = n; }
+      });
     }
     if (has_next) {   // in flight through the pair's end
       if (e_next == e) load_spec(spec, S, s_next);
       else load_spec(evs[e_next].spec, evs[e_next].n_st, s_next);
     }
-    // peak: max value, lowest index on ties
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-      const float ov = __shfl_xor_sync(0xffffffffu, bv, off);
-      const int oi = __shfl_xor_sync(0xffffffffu, bi, off);
-      if (ov > bv || (ov == bv && oi < bi)) { bv = ov; bi = oi; }
-    }
+    // peak: max value, lowest index on ties (values >= 0, or -1 where all are NaN: their bits
+    // compare as integers)
+    const int wtop = __reduce_max_sync(0xffffffffu, __float_as_int(bv));
+    bi = __reduce_min_sync(0xffffffffu, __float_as_int(bv) == wtop ? bi : N);
+    bv = __int_as_float(wtop);
     if ((tid & 31) == 0) { redv[tid >> 5] = bv; redi[tid >> 5] = bi; }
     if (traces) fence_proxy_async_smem();   // each thread's staged writes, visible to the bulk copy
     __syncthreads();
     ++pairs_in_dir;
-    if (tid == 0 && traces) {   // the staged E-field (both components) and envelope to global memory
-      tma_bulk_s2g(ev.efield + pair * 2 * N, stage, 2 * N * sizeof(float));
-      if (wants & kEnvelope) tma_bulk_s2g(ev.envelope + pair * N, stage + 2 * N, N * sizeof(float));
+    // the staged E-field and envelope to global memory: one thread each, with SPLIT == 2 a component
+    // and half of the envelope each
+    if (copies_out && traces) {
+      const int c = tid >> 5;   // 0 or 1
+      if constexpr (SPLIT == 1) {
+        if (c == 0) tma_bulk_s2g(ev.efield + pair * 2 * N, stage, 2 * N * sizeof(float));
+        else if (wants & kEnvelope) tma_bulk_s2g(ev.envelope + pair * N, stage + L::STAGE_V, N * sizeof(float));
+      } else {
+        tma_bulk_s2g(ev.efield + (pair * 2 + c) * N, stage + c * L::STAGE_P, N * sizeof(float));
+        if (wants & kEnvelope)
+          tma_bulk_s2g(ev.envelope + pair * N + c * (N / 2), stage + L::STAGE_V + c * (N / 2 + L::SKEW),
+                       N / 2 * sizeof(float));
+      }
       tma_bulk_commit();
     }
+    const auto env_at = [&](int n) { return stage[L::STAGE_V + n + (n >= N / 2 ? L::SKEW : 0)]; };   // staged
     float snr = 0.f;
-    if (want_snr) {   // every thread takes the pair's peak from the per-warp maxima (as thread 0 does below)
+    if (want_snr) {   // every thread takes the pair's peak from the per-warp maxima (as kPeakLead does below)
       float pv = redv[0];
       int pk = redi[0];
 #pragma unroll
@@ -1323,9 +1331,11 @@ __global__ void __launch_bounds__(Layout<N_>::T, Layout<N_>::MIN_CTAS) unfold_ke
         if (redv[w] > pv || (redv[w] == pv && redi[w] < pk)) { pv = redv[w]; pk = redi[w]; }
       }
       if (pv < 0.f) { pv = 0.f; pk = 0; }
-      snr = pair_snr<T>(stage + 2 * N, N, pk, pv, redw);
+      snr = pair_snr<T, kPeakLead>(env_at, N, pk, pv, redw);
     }
-    if (tid == 0 && pair_ok) {
+    if (tid == kPeakLead && pair_ok) {
+      bv = redv[0];
+      bi = redi[0];
 #pragma unroll
       for (int w = 1; w < T / 32; ++w) {
         if (redv[w] > bv || (redv[w] == bv && redi[w] < bi)) { bv = redv[w]; bi = redi[w]; }
@@ -1335,17 +1345,17 @@ __global__ void __launch_bounds__(Layout<N_>::T, Layout<N_>::MIN_CTAS) unfold_ke
       ev.peak_amp[pair] = bv;   // the peak time is formed with the direction's residual
       if (wants & kFine)
         ev.peak_fine[pair] =
-            __dadd_rn(ev.t_start[s], __dmul_rn(__dadd_rn(static_cast<double>(bi), peak_offset(stage + 2 * N, N, bi)),
+            __dadd_rn(ev.t_start[s], __dmul_rn(__dadd_rn(static_cast<double>(bi), peak_offset(env_at, N, bi)),
                                                ev.dt_ns));
       ev.status[pair] = di.st | (key_sing ? kStSingular : 0u);
       if (want_snr) ev.snr[pair] = snr;
     }
     if (dir_end) {
       // Publish this CTA's pairs of direction d; the last CTA does the residual. One
-      // acquire-release add: it releases thread 0's outputs of the direction (the only ones the
+      // acquire-release add: it releases this thread's outputs of the direction (the only ones the
       // residual reads) and acquires every other CTA's; the barrier passes them on to the
       // CTA's other threads. A direction that lies in this CTA alone needs the barrier only.
-      if (tid == 0) {
+      if (tid == kPeakLead) {
         *sflag = 0;
         if (pair_ok) {
           if (pairs_in_dir == S) {
@@ -1369,7 +1379,7 @@ __global__ void __launch_bounds__(Layout<N_>::T, Layout<N_>::MIN_CTAS) unfold_ke
     s = s_next;
     p = p_next;
   }
-  if (tid == 0) tma_bulk_wait_all();
+  if (copies_out) tma_bulk_wait_all();
 }
 
 // ---- iterative reconstruction (Sec. 2): voltage-maximum timing, plane-wave fit -------------

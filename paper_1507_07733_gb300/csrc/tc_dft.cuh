@@ -545,12 +545,12 @@ __global__ void __launch_bounds__(kSub) tc_inverse_post_kernel(const __grid_cons
     ev.peak_amp[pair] = bv;   // the peak time is formed with the direction's residual
     if (ev.peak_fine)
       ev.peak_fine[pair] =
-          __dadd_rn(ev.t_start[s], __dmul_rn(__dadd_rn(static_cast<double>(bi), peak_offset(senv, N, bi)), ev.dt_ns));
+          __dadd_rn(ev.t_start[s], __dmul_rn(__dadd_rn(static_cast<double>(bi), peak_offset([&](int i) { return senv[i]; }, N, bi)), ev.dt_ns));
   }
   if (ev.snr) {
     __shared__ float rw[kSub / 32];
     __syncthreads();   // the pair's peak visible to every thread
-    const float snr = pair_snr<kSub>(senv, N, pk_i, pk_v, rw);
+    const float snr = pair_snr<kSub, 0>([&](int i) { return senv[i]; }, N, pk_i, pk_v, rw);
     if (n2 == 0) ev.snr[pair] = snr;
   }
 }
