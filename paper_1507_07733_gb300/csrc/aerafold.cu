@@ -14,6 +14,7 @@
 #include <chrono>
 #include <condition_variable>
 #include <deque>
+#include <limits>
 #include <map>
 #include <mutex>
 #include <string>
@@ -475,6 +476,22 @@ EventDesc make_desc(const PathBuffers& b, const ar_pattern_desc& pd, const float
   return d;
 }
 
+// The CTAs of the station kernel that form the direction entries, behind its one per station (at
+// most 256), or 0: a ninth warp of the stations' CTAs forms them. Three of the unfold kernel's CTAs start
+// beside a station CTA of eight warps (1024 and 2048 samples), beside nine warps two, so where the pairs
+// and two places per station exceed the grid the entries have CTAs of their own (2048 samples: 124 x 3
+// pairs 17.1 -> 15.5 us, 30 x 20 18.5 -> 17.2, 124 x 8 21.7 -> 20.6, 124 x 64 73.4 -> 72.4, 113 x 251
+// peaks only 205.3 -> 203.5; with room 10 x 1 11.9 -> 12.1, 124 x 1 13.0 -> 13.4, stays). At 1024 they gain from
+// a quarter of the grid on (124 x 1 11.55 -> 11.2, 124 x 2 12.5 -> 11.9, 101 x 97 53.8 -> 52.3; 10 x 1
+// 10.3 -> 10.5, stays). At 4096 the 72 KB of a station CTA, not its warps, take the place: more
+// CTAs gain nothing (60 x 128 peaks only 144.0 -> 145.0).
+template <int N_>
+int direction_ctas(const EventDesc& ev, long long pairs, int grid_cap) {
+  if (!ev.dir_pre || N_ == 4096 || pairs + 2 * ev.n_st <= (N_ == 1024 ? grid_cap / 4 : grid_cap)) return 0;
+  constexpr int per = SpectrumSmem<N_>::DIRS_PER_CTA;
+  return std::min((ev.n_dir + per - 1) / per, 256);
+}
+
 // The station kernel (one CTA per station) of an event, launched early behind whatever is before
 // it in the stream and waiting for it before it touches anything: its CTAs take their places as the
 // previous call's leave, which saves the launch latency (calls back to back at 2048 samples: 10 x 1
@@ -485,13 +502,15 @@ EventDesc make_desc(const PathBuffers& b, const ar_pattern_desc& pd, const float
 // several pairs per CTA 124 x 5 29.4 -> 27.7): plain stream order there.
 template <int N_>
 cudaError_t launch_station(PathParams pp, long long pairs, int grid_cap, cudaStream_t stream) {
-  const int S = pp.ev0.n_st;
+  using SM = SpectrumSmem<N_>;
+  const int S = pp.ev0.n_st, extra = direction_ctas<N_>(pp.ev0, pairs, grid_cap);
+  const int threads = extra ? SM::THREADS : SM::BLOCK;
   if (Layout<N_>::MIN_CTAS == 2 && pairs <= grid_cap && pairs + S > grid_cap) {
-    station_spectrum_kernel<N_><<<S, SpectrumSmem<N_>::BLOCK, SpectrumSmem<N_>::TOTAL, stream>>>(pp);
+    station_spectrum_kernel<N_><<<S + extra, threads, SM::TOTAL, stream>>>(pp);
     return cudaGetLastError();
   }
   pp.wait_first = 1;
-  return launch_pdl(station_spectrum_kernel<N_>, S, SpectrumSmem<N_>::BLOCK, SpectrumSmem<N_>::TOTAL, stream, pp);
+  return launch_pdl(station_spectrum_kernel<N_>, S + extra, threads, SM::TOTAL, stream, pp);
 }
 
 // One event: the station kernel, then the persistent unfold kernel, launched with programmatic
@@ -511,6 +530,9 @@ cudaError_t launch_path(unsigned* err, const EventDesc& desc, int grid_cap, cuda
   if (evs && (e = cudaEventRecord(evs[0], stream)) != cudaSuccess) return e;
   const long long pairs = static_cast<long long>(desc.n_st) * desc.n_dir;
   if ((e = launch_station<N_>(pp, pairs, grid_cap, stream)) != cudaSuccess) return e;
+  const int extra = direction_ctas<N_>(desc, pairs, grid_cap);
+  // a grid that fills the GPU: each CTA of the station kernel takes the place of one of the unfold kernel's
+  pp.n_early = extra && pairs > grid_cap ? grid_cap - desc.n_st - extra : std::numeric_limits<int>::max();
   if (evs && (e = cudaEventRecord(evs[1], stream)) != cudaSuccess) return e;
   const long long grid = std::min<long long>(grid_cap, pairs);
   const size_t smem = UnfoldSmem<N_>::total(pp.ev0.n_f_layout, pp.ev0.slab_direct != 0);
@@ -1268,6 +1290,7 @@ PathParams batch_params(ar_batch* b, int c, int wait_prior) {
   pp.batch = reinterpret_cast<const BatchHeader*>(b->d_desc[c]);
   pp.err = b->ctx->d_err;
   pp.wait_prior = wait_prior;
+  pp.n_early = std::numeric_limits<int>::max();
   return pp;
 }
 

@@ -243,6 +243,7 @@ struct PathParams {
   unsigned* err;              // device error word
   const int* skip;            // if not null and *skip != 0 the kernel does nothing (a loop has converged)
   int wait_prior;             // wait for the previous kernel in the stream (its results are needed)
+  int n_early;                // unfold CTAs below this index build their first inverse before that wait
   int wait_first;             // (station kernel) wait for it before anything else: launched early behind any kernel
   // Test of the bounded-wait error path (ar_set_test_fault): nonzero makes every corner-slab
   // mbarrier expect 16 bytes more than its four bulk copies deliver, and its waits give up
@@ -332,6 +333,7 @@ struct SpectrumSmem {
   static constexpr int N = N_, M = N_ / 4;
   static constexpr int THREADS = 256;                              // the transform's threads
   static constexpr int BLOCK = THREADS + 32;                       // and one warp for the direction entries
+  static constexpr int DIRS_PER_CTA = 8;                           // or CTAs of their own with this many each
   static constexpr size_t X0 = 0;                                  // [4][M] float2 (ping)
   static constexpr size_t X1 = X0 + sizeof(float2) * 4 * M;        // [4][M] float2 (pong)
   static constexpr size_t TW = X1 + sizeof(float2) * 4 * M;        // [M] exp(-2 pi i x / M)
@@ -379,9 +381,21 @@ __global__ void __launch_bounds__(SpectrumSmem<N_>::BLOCK) station_spectrum_kern
   const int tid = threadIdx.x;
   if (prm.wait_first) pdl_wait_prior();
   pdl_launch_dependents();
-  // threads [0, T) transform (their barriers are named barrier 1); the last warp forms the
-  // per-direction entries meanwhile (directions s, s + S, ... of the event for station s)
+  // threads [0, T) transform (their barriers are named barrier 1); a ninth warp, if there is one, forms
+  // the per-direction entries meanwhile (directions s, s + S, ... of the event for station s)
   const auto sync = [] { asm volatile("bar.sync 1, %0;" ::"n"(SM::THREADS) : "memory"); };
+  if (!prm.batch && static_cast<int>(blockIdx.x) >= prm.ev0.n_st) {
+    // CTAs behind the stations' (a plain launch): direction entries, by one warp in eight slots of
+    // four lanes (FP64 work, 4 us for one direction or eight)
+    if (tid >= 32) return;
+    const int D = prm.ev0.n_dir, S = prm.ev0.n_st;
+    const int stride = (static_cast<int>(gridDim.x) - S) * SM::DIRS_PER_CTA;
+    for (int base = (static_cast<int>(blockIdx.x) - S) * SM::DIRS_PER_CTA; base < D; base += stride) {   // warp-uniform
+      const int d = base + (tid >> 2);
+      precompute_direction(prm.ev0, d, tid & 3, d < D);
+    }
+    return;
+  }
   // a plain launch has one CTA per station; a batch launch walks the stations grid-stride
   const int total = prm.batch ? prm.batch->total_stations : prm.ev0.n_st;
   for (int gs = blockIdx.x; gs < total; gs += gridDim.x) {
@@ -1064,10 +1078,14 @@ __global__ void __launch_bounds__(Layout<N_>::T, Layout<N_>::MIN_CTAS) unfold_ke
   // The station spectra and the walk order come from an earlier kernel; the pattern,
   // directions and station ids do not, unless a skip flag (written by the previous kernel,
   // which may cancel the whole launch) marks a loop whose directions the previous kernel
-  // computes. Without either, the first key's inverse is built before waiting for the
-  // previous kernel. After the wait the next kernel in the stream may launch, so that a kernel
-  // launched behind this one may rely on everything this one waited for.
-  const bool early = prm.skip == nullptr && evs[e0].st_walk == nullptr;
+  // computes. Without either, the first key's inverse is built before waiting for the previous
+  // kernel, its direction cell formed here (FP64 work, 3.5 us by one thread), by the CTAs that start
+  // beside the station kernel. Those that start as its CTAs leave (n_early on) take the cell that
+  // it formed: in a scan of 124 x 64 pairs of 2048 samples they were ready at 14 us, the others at
+  // 9, and ended last (73.2 -> 72.45 us). After the wait the next kernel in the stream may
+  // launch, so that a kernel launched behind this one may rely on everything this one waited for.
+  const bool early =
+      static_cast<int>(blockIdx.x) < prm.n_early && prm.skip == nullptr && evs[e0].st_walk == nullptr;
   if (!early) {
     if (prm.wait_prior) pdl_wait_prior();
     pdl_launch_dependents();

@@ -21,6 +21,7 @@ def _dev(a):
 @pytest.mark.parametrize("n,s,d,n_freq", [
     (1024, 1, 1, 2), (1024, 5, 3, 193), (1024, 4, 2, 256), (1024, 23, 53, 51),
     (2048, 1, 1, 192), (2048, 3, 2, 256), (2048, 29, 21, 51),
+    (1024, 1, 2300, 51), (2048, 57, 9, 51), (2048, 61, 11, 51),   # direction entries by CTAs of their own
     (4096, 1, 2, 256), (4096, 1, 306, 51), (4096, 61, 5, 98),
 ])
 def test_edges_match_the_oracle(n, s, d, n_freq):
