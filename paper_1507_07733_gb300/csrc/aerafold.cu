@@ -236,7 +236,7 @@ ar_status get_pattern_refs(ar_ctx* ctx, int n, double fs, int k_lo, const Patter
       ar_status st = get_bin_table(ctx, n, fs, i, k_lo, &binf);
       if (st != AR_OK) return st;
       refs[i] = PatternRef{ctx->patterns[i].table, binf, pd.zen0_rad, pd.dzen_rad, pd.az0_rad, pd.daz_rad,
-                           pd.n_zen, pd.n_az, pd.n_freq, 0};
+                           reciprocal_of(pd.dzen_rad), reciprocal_of(pd.daz_rad), pd.n_zen, pd.n_az, pd.n_freq, 0};
     }
     PatternRef* d = nullptr;
     AR_CUDA(ctx, cudaMalloc(&d, refs.size() * sizeof(PatternRef)));
@@ -461,6 +461,8 @@ EventDesc make_desc(const PathBuffers& b, const ar_pattern_desc& pd, const float
   d.dzen = pd.dzen_rad;
   d.az0 = pd.az0_rad;
   d.daz = pd.daz_rad;
+  d.inv_dzen = reciprocal_of(pd.dzen_rad);
+  d.inv_daz = reciprocal_of(pd.daz_rad);
   d.dt_ns = 1e9 / ev->fs_hz;
   d.n_over_c = (ev->refractive_index > 0.0 ? ev->refractive_index : 1.0) / kCMPerNs;
   d.inv_n_st = 1.0 / static_cast<double>(ev->n_stations);
@@ -790,7 +792,7 @@ cudaError_t launch_recon(ar_ctx* ctx, const ar_event* ev, int max_iter, double t
   fp.st = st;
   fp.dir_pre = ctx->dir_pre;
   fp.pattern = PatternRef{pat.table, rs.binf, pat.desc.zen0_rad, pat.desc.dzen_rad, pat.desc.az0_rad,
-                          pat.desc.daz_rad, pat.desc.n_zen, pat.desc.n_az, pat.desc.n_freq, 0};
+                          pat.desc.daz_rad, reciprocal_of(pat.desc.dzen_rad), reciprocal_of(pat.desc.daz_rad), pat.desc.n_zen, pat.desc.n_az, pat.desc.n_freq, 0};
   fp.own_pattern = ev->station_pattern ? 0 : 1;
   fp.direction = out->direction;
   fp.t0 = out->t0_ns;

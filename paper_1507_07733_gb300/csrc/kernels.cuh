@@ -28,6 +28,7 @@
 #include <cstdint>
 #include <cuda_runtime.h>
 
+#include "cell.h"
 #include "dft.cuh"
 
 namespace aerafold {
@@ -183,6 +184,7 @@ struct PatternRef {
   const float2* table;     // [n_zen][n_az][n_f][4] VEL (c0p0, c0p1, c1p0, c1p1)
   const int2* binf;        // [M]: (.x = frequency cell or -1 outside the band, .y = bits of t_f)
   double zen0, dzen, az0, daz;
+  double inv_dzen, inv_daz;   // reciprocal_of(dzen), (daz)
   int n_zen, n_az, n_f, pad;
 };
 
@@ -217,7 +219,7 @@ struct EventDesc {
   const PatternRef* pats;  // with st_pat: the loaded patterns at this (N, fs), by pattern id
   const int* st_pat;       // [S] pattern id per station, or null: every station uses the fields here
   int2* st_walk;           // [S] with st_pat: (station, pattern index) in walk order, written by the station kernel
-  double zen0, dzen, az0, daz, dt_ns, n_over_c;
+  double zen0, dzen, az0, daz, inv_dzen, inv_daz, dt_ns, n_over_c;
   double inv_n_st;         // 1 / n_st (FP64, from the host): the fit's mean as a product
   long long pair_begin;    // first pair of the event in the launch's flattened pair space
   int station_begin;       // first station of the event in the launch's flattened station space
@@ -300,6 +302,8 @@ __device__ __forceinline__ PatternRef pattern_ref(const EventDesc& ev, int p) {
   r.dzen = ev.dzen;
   r.az0 = ev.az0;
   r.daz = ev.daz;
+  r.inv_dzen = ev.inv_dzen;
+  r.inv_daz = ev.inv_daz;
   r.n_zen = ev.n_zen;
   r.n_az = ev.n_az;
   r.n_f = ev.n_f;
@@ -365,11 +369,12 @@ __device__ __forceinline__ void stockham_stage(const float2* __restrict__ in, fl
 // a part of direction d's per-direction entry (defined with the cells)
 __device__ void precompute_direction(const EventDesc& ev, int d, int part, bool valid);
 
-// One CTA per station of the launch. x[4m + r] (both channels packed as v0 + i v1) -> four
+// One CTA per station of the launch, in at most 56 registers (8 warps of more and only two of the unfold
+// kernel's CTAs start beside it). x[4m + r] (both channels packed as v0 + i v1) -> four
 // M-point DFTs U_r by three Stockham stages, then Z[k] = sum_r W_N^{kr} U_r[k mod M] at the
 // band bins and the split into the two channels' spectra.
 template <int N_>
-__global__ void __launch_bounds__(SpectrumSmem<N_>::BLOCK) station_spectrum_kernel(const __grid_constant__ PathParams prm) {
+__global__ void __launch_bounds__(SpectrumSmem<N_>::BLOCK, 4) station_spectrum_kernel(const __grid_constant__ PathParams prm) {
   using SM = SpectrumSmem<N_>;
   using RD = StationRadix<N_>;
   constexpr int N = N_, M = SM::M, T = SM::THREADS;
@@ -386,7 +391,7 @@ __global__ void __launch_bounds__(SpectrumSmem<N_>::BLOCK) station_spectrum_kern
   const auto sync = [] { asm volatile("bar.sync 1, %0;" ::"n"(SM::THREADS) : "memory"); };
   if (!prm.batch && static_cast<int>(blockIdx.x) >= prm.ev0.n_st) {
     // CTAs behind the stations' (a plain launch): direction entries, by one warp in eight slots of
-    // four lanes (FP64 work, 4 us for one direction or eight)
+    // four lanes (FP64 work, 3 us for one direction or eight)
     if (tid >= 32) return;
     const int D = prm.ev0.n_dir, S = prm.ev0.n_st;
     const int stride = (static_cast<int>(gridDim.x) - S) * SM::DIRS_PER_CTA;
@@ -505,36 +510,13 @@ struct DirPre {
   double pad;
 };
 
-// Direction -> pattern cell (FP64, no fused multiply-adds) -> FP32 bilinear weights, in two
-// halves that different lanes can form (FP64 is slow here: a chain of two divisions and one of
-// one take less time side by side).
-//
-// The azimuth's position in the table's steps, reduced to [0, n_az]; false if it has none. An
-// azimuth has a place when it is finite and less than 2^52 azimuth steps from az0 (beyond, one
-// FP64 unit is a whole step). Below that bound the remainder modulo n_az lands in [0, n_az]; the
-// range test keeps every slab index in bounds.
-__device__ __forceinline__ bool azimuth_position(const PatternRef& p, double az, double* ua_out) {
-  double ua = 0.0;
-  bool ok = isfinite(az);
-  if (ok) {
-    ua = __ddiv_rn(__dsub_rn(az, p.az0), p.daz);
-    ok = fabs(ua) < 0x1p52;
-  }
-  if (ok) {
-    ua = __dsub_rn(ua, __dmul_rn(double(p.n_az), floor(__ddiv_rn(ua, double(p.n_az)))));
-    ok = ua >= 0.0 && ua <= double(p.n_az);
-  }
-  *ua_out = ua;
-  return ok;
+// Direction -> pattern cell (FP64) -> FP32 bilinear weights, in two halves that different lanes can
+// form: the azimuth's position in the table's steps and the zenith's.
+__device__ __forceinline__ bool azimuth_position(const PatternRef& p, double az, double* ua) {
+  return azimuth_place(divide_by(__dsub_rn(az, p.az0), p.daz, p.inv_daz), az, p.n_az, ua);
 }
-// The zenith's position, clamped to [0, n_zen - 1] (*clamped); false if it is not finite.
-__device__ __forceinline__ bool zenith_position(const PatternRef& p, double zen, double* uz_out, bool* clamped) {
-  double uz = __ddiv_rn(__dsub_rn(zen, p.zen0), p.dzen);
-  *clamped = false;
-  if (uz < 0.0) { uz = 0.0; *clamped = true; }
-  if (uz > double(p.n_zen - 1)) { uz = double(p.n_zen - 1); *clamped = true; }
-  *uz_out = uz;
-  return isfinite(zen);
+__device__ __forceinline__ bool zenith_position(const PatternRef& p, double zen, double* uz, bool* clamped) {
+  return zenith_place(divide_by(__dsub_rn(zen, p.zen0), p.dzen, p.inv_dzen), zen, p.n_zen, uz, clamped);
 }
 __device__ __forceinline__ DirInfo cell_of_positions(const PatternRef& p, bool has_cell, double uz, bool clamped,
                                                      double ua) {
@@ -848,11 +830,12 @@ __device__ void precompute_direction(const EventDesc& ev, int d, int part, bool 
   const PatternRef pr = pattern_ref(ev, -1);
   if (valid && (part == 1 || part == 2)) {
     sincos(ev.dirs[2 * d + (part - 1)], &sv, &cv);
-  } else if (valid && cell && part == 0) {
-    flags = azimuth_position(pr, ev.dirs[2 * d + 1], &sv) ? 1 : 0;
   } else if (valid && cell) {
-    bool clamped;
-    flags = zenith_position(pr, ev.dirs[2 * d], &sv, &clamped) ? 1 : 0;
+    const bool az = part == 0;   // one division for both (diverged lanes take turns)
+    const double x = ev.dirs[2 * d + (az ? 1 : 0)];
+    const double steps = divide_by(__dsub_rn(x, az ? pr.az0 : pr.zen0), az ? pr.daz : pr.dzen, az ? pr.inv_daz : pr.inv_dzen);
+    bool clamped = false;
+    flags = (az ? azimuth_place(steps, x, pr.n_az, &sv) : zenith_place(steps, x, pr.n_zen, &sv, &clamped)) ? 1 : 0;
     flags |= clamped ? 2 : 0;
   }
   // part 1 (zenith) takes the azimuth's sine and cosine from part 2, part 0 the zenith from part 3
@@ -1079,7 +1062,7 @@ __global__ void __launch_bounds__(Layout<N_>::T, Layout<N_>::MIN_CTAS) unfold_ke
   // directions and station ids do not, unless a skip flag (written by the previous kernel,
   // which may cancel the whole launch) marks a loop whose directions the previous kernel
   // computes. Without either, the first key's inverse is built before waiting for the previous
-  // kernel, its direction cell formed here (FP64 work, 3.5 us by one thread), by the CTAs that start
+  // kernel, its direction cell formed here (FP64 work by one thread), by the CTAs that start
   // beside the station kernel. Those that start as its CTAs leave (n_early on) take the cell that
   // it formed: in a scan of 124 x 64 pairs of 2048 samples they were ready at 14 us, the others at
   // 9, and ended last (73.2 -> 72.45 us). After the wait the next kernel in the stream may
