@@ -1084,10 +1084,13 @@ __global__ void __launch_bounds__(Layout<N_>::T, Layout<N_>::MIN_CTAS) unfold_ke
     mbar_init(bar, 1);
     issue_key(evs[e0], d, p, sdir, slab, bar, !early, prm.err, prm.test_wait ? 16u : 0u);
   }
+  // the first event's descriptor into shared memory meanwhile (behind the cell and its slabs: 10 x 1
+  // pairs of 2048 samples 10.9 -> 10.65 us, 124 x 64 72.0 -> 71.55, 113 x 251 peaks 202.6 -> 200.9)
+  if (tid >= 32) copy_event(sev, evs + e0, tid - 32, T - 32);
   bool pending = slab_staged(evs[e0], p);   // slab copies to wait for before the next build
-  __syncthreads();    // barrier initialised, first direction cell visible
+  __syncthreads();    // barrier initialised, first direction cell and event visible
 
-  bool new_event = true, new_key = true;   // of the pair at hand
+  bool new_event = false, new_key = true;   // of the pair at hand
   int run = 0;               // pairs that follow it in this CTA with the next station of the same key
   int S = 0;                 // the event's stations, spectra and outputs asked for
   const float4* spec = nullptr;
@@ -1108,6 +1111,14 @@ __global__ void __launch_bounds__(Layout<N_>::T, Layout<N_>::MIN_CTAS) unfold_ke
 #pragma unroll
     for (int i = 0; i < NB; ++i) vin[i] = __ldcg(src + T * i);
   };
+  const auto event_facts = [&]() {   // of the event in sev
+    const EventDesc& ev = *sev;
+    S = ev.n_st;
+    spec = ev.spec;
+    wants = (ev.efield ? kTraces : 0u) | (ev.efield && ev.envelope ? kEnvelope : 0u) |
+            (ev.peak_fine ? kFine : 0u) | (kSnr && ev.snr ? kWantSnr : 0u) | (ev.st_walk ? kWalk : 0u);
+  };
+  event_facts();
   for (int q = 0;; ++q) {
     const EventDesc& ev = *sev;
     if (new_key) {
@@ -1128,10 +1139,7 @@ __global__ void __launch_bounds__(Layout<N_>::T, Layout<N_>::MIN_CTAS) unfold_ke
       if (new_event) {   // its descriptor into shared memory
         copy_event(sev, evs + e, tid, T);
         __syncthreads();
-        S = ev.n_st;
-        spec = ev.spec;
-        wants = (ev.efield ? kTraces : 0u) | (ev.efield && ev.envelope ? kEnvelope : 0u) |
-                (ev.peak_fine ? kFine : 0u) | (kSnr && ev.snr ? kWantSnr : 0u) | (ev.st_walk ? kWalk : 0u);
+        event_facts();
       }
       // the inverse of every bin, shared by the key's stations. The node scratch overlays A: the
       // previous pair's staged outputs must have left it.
