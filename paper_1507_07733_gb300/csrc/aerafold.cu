@@ -1105,11 +1105,13 @@ cudaError_t launch_gemm(ar_ctx* ctx, __nv_bfloat16* const (&a)[3], size_t m_pad,
   gp.terms = terms;
   int groups = 1;
   const int tiles128 = static_cast<int>(m_pad / tc::kBM) * (n / tc::kBN);
-  while (groups * 2 <= gp.chunks && tiles128 * groups * 2 <= 2 * ctx->num_sms) groups *= 2;
+  while (groups * 4 <= gp.chunks && tiles128 * groups * 2 <= 2 * ctx->num_sms) groups *= 2;
   gp.chunks_per_group = gp.chunks / groups;
-  // 256-wide tiles (half the MMA instructions and B-operand copies per flop) for the two-plane
-  // split when every item is a single fold unit of at most four chunks and enough tiles remain
-  const bool wide = terms == 3 && gp.chunks_per_group <= 4 && n % 256 == 0 &&
+  // 256-wide tiles when every item is a single fold unit and at least two tiles per SM remain. At width 128
+  // an MMA's operands (8 KB in 64 cycles) take all of shared memory's bandwidth and the stages' copies
+  // slow it; at 256 (12 KB in 128) there is room for them: x6 at 43 x 29 pairs of 4096 samples 125.2 ->
+  // 119.3 us the call, at 124 x 64 of 2048 288.0 -> 265.4.
+  const bool wide = gp.chunks_per_group <= tc::kFoldChunks && n % 256 == 0 &&
                     static_cast<long long>(m_pad / tc::kBM) * (n / 256) >= 2 * ctx->num_sms;
   const int bn = wide ? 256 : tc::kBN;
   const int tiles = static_cast<int>(m_pad / tc::kBM) * (n / bn);

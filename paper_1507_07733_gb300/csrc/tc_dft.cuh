@@ -25,16 +25,16 @@
 //
 // Tensor-core details (PTX ISA, tcgen05). A persistent CTA (one per SM) computes 128 x 128
 // tiles of D = A B^T (A row-major M x K, B row-major N x K, both K-major), each over a range
-// of 64-wide K chunks, with 6 warps in three roles: warp 4 stages each chunk's operands with bulk copies into one of two
-// shared-memory stages (mbarrier full/empty pairs), warp 5 issues the tcgen05.mma
+// of 32-wide K chunks, with 6 warps in three roles: warp 4 stages each chunk's operands with bulk copies into a ring of
+// three to six shared-memory stages (mbarrier full/empty pairs), warp 5 issues the tcgen05.mma
 // instructions (M 128, N 128, K 16; one per split product and K step) into tensor memory,
 // and warps 0-3 read the chunk's partial sum out of tensor memory (tcgen05.ld) and fold it
 // into the running sum (see the accumulation note below), writing the result at the end.
 // Every wait is bounded. Operands come pre-split and pre-arranged in the shared-memory image
 // of the no-swizzle K-major core-matrix layout: a core matrix is 8 rows x 16 bytes; in a
-// 128-row, 64-column block the core matrix of rows 8a..8a+7 and columns 8b..8b+7 starts at
-// byte 1024 a + 128 b (leading byte offset 128 along K, stride byte offset 1024 along M or N);
-// one 16 KB block per (row tile, K chunk, plane), so a stage is filled by plain 1-D bulk
+// 128-row, 32-column block the core matrix of rows 8a..8a+7 and columns 8b..8b+7 starts at
+// byte 512 a + 128 b (leading byte offset 128 along K, stride byte offset 512 along M or N);
+// one 8 KB block per (row tile, K chunk, plane), so a stage is filled by plain 1-D bulk
 // copies. The producers of A (the forward pre-pass and the solve) write this image directly.
 #pragma once
 #include <cuda_bf16.h>
@@ -47,24 +47,25 @@ namespace tc {
 
 constexpr int kSub = 512;                         // sub-block length
 constexpr int kBandPhase = 128;                   // band bins per sub-block phase j1 (M / A)
-constexpr int kBM = 128, kBN = 128, kBK = 64;     // CTA tile and K chunk
+constexpr int kBM = 128, kBN = 128, kBK = 32;     // CTA tile and K chunk
+constexpr int kFoldChunks = 8;                    // chunks accumulated on the tensor cores between folds, at most
 constexpr unsigned kErrBadLaunch = 2u;           // device error bit: a launch configuration the GEMM does not take
-constexpr unsigned kBlk = kBM * kBK * 2;          // bytes of one BF16 plane of a 128 x 64 block (16 KB)
-constexpr unsigned kStageBytes = 6 * kBlk;        // A and B, up to 3 planes each
-constexpr int kStages = 2;                          // ring bytes: 2 such stages (x6) or 3 of 4 blocks (x3)
+constexpr unsigned kBlk = kBM * kBK * 2;          // bytes of one BF16 plane of a 128 x 32 block (8 KB)
+constexpr unsigned kRingBytes = 27 * kBlk;        // the stage ring (216 KB): three stages of the largest kind
+constexpr int kMaxStages = 6;
 constexpr int kFwdK = 2 * kSub, kFwdN = 2 * kBandPhase;   // forward GEMM: K 1024, 256 outputs
 constexpr int kInvK = 2 * kBandPhase, kInvN = 2 * kSub;   // inverse GEMM: K 256, 1024 outputs
-constexpr size_t kEpiBytes = 4 * 32 * 32 * sizeof(float);   // a 32 x 32 transpose tile per fold warp
-constexpr size_t kGemmSmem = kStages * kStageBytes + 256 + kEpiBytes;
+constexpr size_t kEpiBytes = 4 * 32 * 16 * sizeof(float);   // a 32 x 16 transpose tile per fold warp
+constexpr size_t kGemmSmem = kRingBytes + 256 + kEpiBytes;
 constexpr int kGemmThreads = 192;
 
-// byte offset of element (r, c) inside a 128-row, 64-column K-major BF16 block
+// byte offset of element (r, c) inside a 128-row, 32-column K-major BF16 block
 __host__ __device__ constexpr unsigned core_offset(int r, int c) {
-  return static_cast<unsigned>((r >> 3) * 1024 + (c >> 3) * 128 + (r & 7) * 16 + (c & 7) * 2);
+  return static_cast<unsigned>((r >> 3) * (kBK * 16) + (c >> 3) * 128 + (r & 7) * 16 + (c & 7) * 2);
 }
-// BF16 element offset of (row, k) in an image of rows x k (blocks [row / 128][k / 64])
+// BF16 element offset of (row, k) in an image of rows x k (blocks [row / 128][k / 32])
 __host__ __device__ constexpr size_t image_offset(int row, int k, int k_total) {
-  return (static_cast<size_t>(row >> 7) * (k_total >> 6) + (k >> 6)) * (kBlk / 2) + core_offset(row & 127, k & 63) / 2;
+  return (static_cast<size_t>(row >> 7) * (k_total / kBK) + k / kBK) * (kBlk / 2) + core_offset(row & 127, k % kBK) / 2;
 }
 
 // instruction descriptor of tcgen05.mma kind::f16: D FP32 (bits 4-5 = 1), A and B BF16
@@ -78,7 +79,7 @@ __host__ __device__ constexpr uint32_t idesc() {
 // (bits 16-29), stride byte offset >> 4 (bits 32-45), version 1 (bits 46-47), no swizzle
 __device__ __forceinline__ uint64_t smem_desc(const void* p) {
   const uint64_t a = smem_u32(p);
-  return ((a & 0x3FFFFull) >> 4) | (uint64_t(128 >> 4) << 16) | (uint64_t(1024 >> 4) << 32) | (1ull << 46);
+  return ((a & 0x3FFFFull) >> 4) | (uint64_t(128 >> 4) << 16) | (uint64_t((kBK * 16) >> 4) << 32) | (1ull << 46);
 }
 
 // the products kept, as (plane of A, plane of B), most significant first
@@ -86,7 +87,7 @@ __device__ __forceinline__ uint64_t smem_desc(const void* p) {
 __host__ __device__ constexpr int term_a(int t) { return t == 2 || t == 4 ? 1 : t == 5 ? 2 : 0; }
 __host__ __device__ constexpr int term_b(int t) { return t == 1 || t == 4 ? 1 : t == 3 ? 2 : 0; }
 
-// The MMAs of one 64-wide K chunk held in the stage whose descriptor is base (A planes of
+// The MMAs of one 32-wide K chunk held in the stage whose descriptor is base (A planes of
 // 128 rows, then B planes of BN rows): for each 16-wide K step every kept product,
 // accumulating into dst except at the first MMA of a fold unit. Unrolled with the terms
 // fixed, so each MMA's descriptors are the base plus a constant.
@@ -111,8 +112,8 @@ __device__ __forceinline__ void mma_chunk(uint64_t base, uint32_t dst, bool unit
 }
 
 struct GemmParams {
-  const uint4* a[3];       // BF16 planes of A, image [m_tiles][chunks] of 16 KB blocks
-  const uint4* b[3];       // BF16 planes of B, image [n_tiles][chunks] of 16 KB blocks
+  const uint4* a[3];       // BF16 planes of A, image [m_tiles][chunks] of 8 KB blocks
+  const uint4* b[3];       // BF16 planes of B, image [n_tiles][chunks] of 8 KB blocks
   float* d;                // D, row-major with row stride ldd; split-K group g at d + g * d_group
   size_t d_group;
   unsigned* err;
@@ -187,11 +188,11 @@ __device__ __forceinline__ void tc_commit(uint64_t* bar) {
 
 // Accumulation. The tensor cores' FP32 accumulator loses about 2^-26 of relative precision,
 // with a bias, at every MMA (measured: the error grows linearly with the number of MMAs into
-// one accumulator), so each fold unit (up to four 64-wide K chunks) is accumulated on its own
+// one accumulator), so each fold unit (up to eight 32-wide K chunks) is accumulated on its own
 // into a partial region P[unit % 2] of tensor memory, and warps 0-3 fold it into the running
 // sum S with IEEE round-to-nearest FP32 additions, in order: S = (((P0 + P1) + P2) + ...).
 // With two partial regions the MMAs of one unit overlap the fold of the previous one.
-// BN = 128: S, P0, P1 of 128 columns each; BN = 256 (x3 items of at most four chunks, which
+// BN = 128: S, P0, P1 of 128 columns each; BN = 256 (items of at most eight chunks, which
 // are single fold units and need no S): P0, P1 of 256 columns.
 constexpr int kTmemCols = 512;
 
@@ -200,13 +201,13 @@ __global__ void __launch_bounds__(kGemmThreads, 1) split_gemm_kernel(const __gri
   static_assert(BN == 128 || BN == 256, "tile width");
   constexpr int NB = BN / 128;   // 128-row B blocks per tile
   extern __shared__ __align__(1024) unsigned char smem[];
-  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + kStages * kStageBytes);
-  uint64_t* full = bars;          // [3] stage filled (bulk copies complete)
-  uint64_t* empty = bars + 3;     // [3] stage consumed (its MMAs complete)
-  uint64_t* ready = bars + 6;     // [2] partial region holds a finished chunk
-  uint64_t* pfree = bars + 8;     // [2] partial region folded (4 arrivals, one per fold warp)
-  uint64_t* done = bars + 10;     // every MMA complete
-  uint32_t* taddr_s = reinterpret_cast<uint32_t*>(bars + 11);
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + kRingBytes);
+  uint64_t* full = bars;                  // [kMaxStages] stage filled (bulk copies complete)
+  uint64_t* empty = full + kMaxStages;    // [kMaxStages] stage consumed (its MMAs complete)
+  uint64_t* ready = empty + kMaxStages;   // [2] partial region holds a finished chunk
+  uint64_t* pfree = ready + 2;            // [2] partial region folded (4 arrivals, one per fold warp)
+  uint64_t* done = pfree + 2;             // every MMA complete
+  uint32_t* taddr_s = reinterpret_cast<uint32_t*>(done + 1);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   pdl_launch_dependents();
   const int items = p.m_tiles * p.n_tiles * p.groups;
@@ -217,16 +218,16 @@ __global__ void __launch_bounds__(kGemmThreads, 1) split_gemm_kernel(const __gri
   const int cpg = p.chunks_per_group;
   const int nk = my_items * cpg;
   const int planes = p.terms == 6 ? 3 : 2;
-  // The stage ring in the same 192 KB: three stages of 2 + 2 blocks (x3, BN 128), two of
-  // 3 + 3 (x6, BN 128) or two of 2 + 4 (x3, BN 256).
+  // The stage ring in the same 216 KB: stages of 4 blocks (x3, BN 128), 6 (x6, BN 128; x3, BN 256) or
+  // 9 (x6, BN 256).
   const unsigned stage_bytes = static_cast<unsigned>(planes * (1 + NB)) * kBlk;
-  const int nst = min(3, static_cast<int>(kStages * kStageBytes / stage_bytes));
-  // Chunks per fold: up to 4 (K = 256 accumulated on the tensor cores between folds), a
-  // divisor of the item's chunk count; an item of at most 4 chunks is one fold unit, whose
+  const int nst = min(kMaxStages, static_cast<int>(kRingBytes / stage_bytes));
+  // Chunks per fold: up to 8 (K = 256 accumulated on the tensor cores between folds), a
+  // divisor of the item's chunk count; an item of at most 8 chunks is one fold unit, whose
   // fold only moves the accumulator to global memory.
-  const int F = cpg <= 4 ? cpg : cpg % 4 == 0 ? 4 : cpg % 2 == 0 ? 2 : 1;
+  const int F = cpg <= kFoldChunks ? cpg : cpg % 8 == 0 ? 8 : cpg % 4 == 0 ? 4 : cpg % 2 == 0 ? 2 : 1;
   const int nu = nk / F;   // fold units
-  if (NB == 2 && (F != cpg || planes != 2)) {   // the wide tile has no running sum and room for 2 planes
+  if (NB == 2 && F != cpg) {   // the wide tile has no running sum
     if (tid == 0) atomicOr(p.err, kErrBadLaunch);
     return;
   }
@@ -238,7 +239,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) split_gemm_kernel(const __gri
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   if (tid == 32) {
-    for (int i = 0; i < 11; ++i) mbar_init(bars + i, (i == 8 || i == 9) ? 4 : 1);
+    for (uint64_t* b = bars; b <= done; ++b) mbar_init(b, b == pfree || b == pfree + 1 ? 4 : 1);
   }
   tc_fence_before();
   __syncthreads();
@@ -299,7 +300,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) split_gemm_kernel(const __gri
   } else {
     // ---- fold warps: S = S + P[chunk % 2]; an item's last chunk goes to global memory ----
     const uint32_t lanes = static_cast<uint32_t>(32 * warp) << 16;
-    float4* epi = reinterpret_cast<float4*>(smem + kStages * kStageBytes + 256) + warp * 32 * 8;
+    float4* epi = reinterpret_cast<float4*>(smem + kRingBytes + 256) + warp * 32 * 4;
     for (int u = 0; u < nu; ++u) {
       const int b = u & 1;
       ok = __all_sync(0xffffffffu, mbar_wait_bounded(&ready[b], (u >> 1) & 1, kWaitLimitNs));   // warp-uniform
@@ -325,20 +326,25 @@ __global__ void __launch_bounds__(kGemmThreads, 1) split_gemm_kernel(const __gri
           for (int k = 0; k < 32; ++k) x[k] = __float_as_uint(__fadd_rn(__uint_as_float(y[k]), __uint_as_float(x[k])));
         }
         if (last) {
-          // Lane l holds row l of the warp's 32 x 32 block. Transposed through shared memory
-          // (16-byte chunk j of row r at chunk j ^ (r & 7): both sides free of bank conflicts)
-          // so that each store instruction writes four rows of 128 contiguous bytes.
+          // Lane l holds row l of the warp's 32 x 32 block. Transposed in two halves through shared
+          // memory (16-byte chunk j of row r at chunk j ^ ((r >> 1) & 3): both sides free of bank
+          // conflicts) so that each store instruction writes eight rows of 64 contiguous bytes.
 #pragma unroll
-          for (int j = 0; j < 8; ++j)
-            epi[lane * 8 + (j ^ (lane & 7))] = make_float4(__uint_as_float(x[4 * j]), __uint_as_float(x[4 * j + 1]),
-                                                           __uint_as_float(x[4 * j + 2]), __uint_as_float(x[4 * j + 3]));
-          __syncwarp();
+          for (int hf = 0; hf < 2; ++hf) {
 #pragma unroll
-          for (int i = 0; i < 8; ++i) {
-            const int r = 4 * i + (lane >> 3), ch = lane & 7;
-            *reinterpret_cast<float4*>(drow + static_cast<size_t>(r) * p.ldd + c + 4 * ch) = epi[r * 8 + (ch ^ (r & 7))];
+            for (int j = 0; j < 4; ++j)
+              epi[lane * 4 + (j ^ ((lane >> 1) & 3))] =
+                  make_float4(__uint_as_float(x[16 * hf + 4 * j]), __uint_as_float(x[16 * hf + 4 * j + 1]),
+                              __uint_as_float(x[16 * hf + 4 * j + 2]), __uint_as_float(x[16 * hf + 4 * j + 3]));
+            __syncwarp();
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+              const int r = 8 * i + (lane >> 2), ch = lane & 3;
+              *reinterpret_cast<float4*>(drow + static_cast<size_t>(r) * p.ldd + c + 16 * hf + 4 * ch) =
+                  epi[r * 4 + (ch ^ ((r >> 1) & 3))];
+            }
+            __syncwarp();   // the tile is read before the next half overwrites it
           }
-          __syncwarp();   // the tile is read before the next block overwrites it
         } else {
           tmem_st32(t_sum + lanes + c, x);
         }
