@@ -1049,10 +1049,10 @@ ar_status build_tc_tables(ar_ctx* ctx) {
       AR_CUDA(ctx, cudaMemcpy(ctx->tc_b[which][pl], img[pl].data(), bytes, cudaMemcpyHostToDevice));
     }
   }
-  AR_CUDA(ctx, cudaFuncSetAttribute(tc::split_gemm_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    static_cast<int>(tc::kGemmSmem)));
-  AR_CUDA(ctx, cudaFuncSetAttribute(tc::split_gemm_kernel<256>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    static_cast<int>(tc::kGemmSmem)));
+  for (auto* kernel : {tc::split_gemm_kernel<128>, tc::split_gemm_kernel<256>, tc::split_gemm_kernel<256, 2>,
+                       tc::split_gemm_kernel<256, 4>, tc::split_gemm_kernel<256, 8>})
+    AR_CUDA(ctx, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      static_cast<int>(tc::kGemmSmem)));
   return AR_OK;
 }
 
@@ -1087,12 +1087,23 @@ TcWorkspace tc_layout(unsigned char* base, size_t rows_f, size_t rows_c, int num
   return w;
 }
 
+// The groups that K is split into: 1 where there are more 128 x 128 tiles than SMs, else up to 64-wide ones.
+int gemm_groups(size_t m_pad, int which, int num_sms) {
+  const int k = which == 0 ? tc::kFwdK : tc::kInvK, n = which == 0 ? tc::kFwdN : tc::kInvN;
+  const int tiles = static_cast<int>(m_pad / tc::kBM) * (n / tc::kBN);
+  int groups = 1;
+  while (groups * 128 <= k && tiles * groups * 2 <= 2 * num_sms) groups *= 2;
+  return groups;
+}
+
 // D (m_pad x n) = A (m_pad x K, image planes) B^T on the tensor cores. When the grid of output
 // tiles is small, K is split into groups whose folded partial sums a second kernel adds in
 // group order.
+// With post (its fields of the parameters) the inverse GEMM of traces of 512 A samples forms the outputs itself
+// instead of D where K is not split (see gemm_groups).
 cudaError_t launch_gemm(ar_ctx* ctx, __nv_bfloat16* const (&a)[3], size_t m_pad, int which, int terms, float* d,
-                        float* part, cudaStream_t stream) {
-  tc::GemmParams gp{};
+                        float* part, cudaStream_t stream, const tc::GemmParams* post = nullptr, int A = 0) {
+  tc::GemmParams gp = post ? *post : tc::GemmParams{};
   const int k = which == 0 ? tc::kFwdK : tc::kInvK;
   const int n = which == 0 ? tc::kFwdN : tc::kInvN;
   for (int pl = 0; pl < 3; ++pl) {
@@ -1103,16 +1114,15 @@ cudaError_t launch_gemm(ar_ctx* ctx, __nv_bfloat16* const (&a)[3], size_t m_pad,
   gp.ldd = n;
   gp.chunks = k / tc::kBK;
   gp.terms = terms;
-  int groups = 1;
-  const int tiles128 = static_cast<int>(m_pad / tc::kBM) * (n / tc::kBN);
-  while (groups * 4 <= gp.chunks && tiles128 * groups * 2 <= 2 * ctx->num_sms) groups *= 2;
+  const int groups = gemm_groups(m_pad, which, ctx->num_sms);
+  if (groups > 1) post = nullptr;
   gp.chunks_per_group = gp.chunks / groups;
   // 256-wide tiles when every item is a single fold unit and at least two tiles per SM remain. At width 128
   // an MMA's operands (8 KB in 64 cycles) take all of shared memory's bandwidth and the stages' copies
   // slow it; at 256 (12 KB in 128) there is room for them: x6 at 43 x 29 pairs of 4096 samples 125.2 ->
   // 119.3 us the call, at 124 x 64 of 2048 288.0 -> 265.4.
-  const bool wide = gp.chunks_per_group <= tc::kFoldChunks && n % 256 == 0 &&
-                    static_cast<long long>(m_pad / tc::kBM) * (n / 256) >= 2 * ctx->num_sms;
+  const bool wide = post || (gp.chunks_per_group <= tc::kFoldChunks && n % 256 == 0 &&
+                             static_cast<long long>(m_pad / tc::kBM) * (n / 256) >= 2 * ctx->num_sms);
   const int bn = wide ? 256 : tc::kBN;
   const int tiles = static_cast<int>(m_pad / tc::kBM) * (n / bn);
   gp.d = groups > 1 ? part : d;
@@ -1122,7 +1132,11 @@ cudaError_t launch_gemm(ar_ctx* ctx, __nv_bfloat16* const (&a)[3], size_t m_pad,
   gp.groups = groups;
   // persistent: one CTA per SM (the kernel's shared memory allows one), items strided
   const int items = tiles * groups;
-  cudaError_t e = launch_pdl(wide ? tc::split_gemm_kernel<256> : tc::split_gemm_kernel<128>,
+  cudaError_t e = launch_pdl(post && A == 2   ? tc::split_gemm_kernel<256, 2>
+                             : post && A == 4 ? tc::split_gemm_kernel<256, 4>
+                             : post           ? tc::split_gemm_kernel<256, 8>
+                             : wide           ? tc::split_gemm_kernel<256>
+                                              : tc::split_gemm_kernel<128>,
                              std::min(items, ctx->num_sms), tc::kGemmThreads, tc::kGemmSmem, stream, gp);
   if (e != cudaSuccess || groups == 1) return e;
   const size_t n4 = gp.d_group / 4;
@@ -1158,6 +1172,21 @@ cudaError_t launch_tc(ar_ctx* ctx, const EventDesc& ev, int terms, size_t rows_f
   if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&solve_per_sm, tc::tc_solve_kernel<N_>, tc::kSolveThreads,
                                                          solve_smem)) != cudaSuccess)
     return e;
+  // The inverse GEMM forms the outputs itself unless one needs a pair's whole envelope, or K is split (few pairs: their
+  // partial sums are added in FP32 first). Measured at 4096 samples, x6: 20 x 10 pairs 49.1 -> 42.3 us, 30 x 20 71.8 ->
+  // 54.9, 43 x 29 119 -> 94.6; at 2048 20 x 20 45.1 -> 40.0, 124 x 64 266 -> 186; at 1024 40 x 20 44.3 -> 39.9.
+  // The peaks' words take the place of the forward GEMM's A image.
+  tc::GemmParams post{};
+  post.wn = ev.wn;
+  post.efield = ev.efield;
+  post.envelope = ev.envelope;
+  post.k_lo = ev.k_lo;
+  const auto unsplit = [&](long long np) {
+    return gemm_groups(pad128(static_cast<size_t>(2 * A) * np), 1, ctx->num_sms) == 1;
+  };
+  if (!ev.peak_fine && !ev.snr && unsplit(std::min(chunk, pairs)) &&
+      static_cast<size_t>(pairs) * sizeof(unsigned long long) <= planes * rows_f * tc::kFwdK * sizeof(__nv_bfloat16))
+    post.peaks = reinterpret_cast<unsigned long long*>(w.fa[0]);
   const long long solve_slots = std::max(1, solve_per_sm) * static_cast<long long>(ctx->num_sms);
   for (long long p0 = 0; p0 < pairs; p0 += chunk) {
     const int np = static_cast<int>(std::min(chunk, pairs - p0));
@@ -1166,17 +1195,21 @@ cudaError_t launch_tc(ar_ctx* ctx, const EventDesc& ev, int terms, size_t rows_f
     const int ppc = static_cast<int>(
         std::max<long long>(1, std::min<long long>(tc::kSolvePairsMax, (np + solve_slots - 1) / solve_slots)));
     tc::tc_solve_kernel<N_><<<(np + ppc - 1) / ppc, tc::kSolveThreads, solve_smem, stream>>>(
-        ev, reinterpret_cast<const float2*>(w.xf), zimg, p0, np, ppc);
+        ev, reinterpret_cast<const float2*>(w.xf), zimg, p0, np, ppc, post.peaks);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if (prof && p0 == 0 && (e = cudaEventRecord(ctx->ev[1], stream)) != cudaSuccess) return e;
-    if ((e = launch_gemm(ctx, w.za, pad128(static_cast<size_t>(2 * A) * np), 1, terms, w.yi, w.part, stream)) !=
-        cudaSuccess)
+    post.pair0 = p0;
+    post.n_pairs = np;
+    if ((e = launch_gemm(ctx, w.za, pad128(static_cast<size_t>(2 * A) * np), 1, terms, w.yi, w.part, stream,
+                         post.peaks ? &post : nullptr, A)) != cudaSuccess)
       return e;
     if (prof && p0 == 0 && (e = cudaEventRecord(ctx->ev[2], stream)) != cudaSuccess) return e;
-    tc::tc_inverse_post_kernel<N_><<<np, tc::kSub, 0, stream>>>(ev, reinterpret_cast<const float2*>(w.yi), p0);
+    if (post.peaks && unsplit(np)) continue;
+    tc::tc_inverse_post_kernel<N_><<<np, tc::kSub, 0, stream>>>(ev, reinterpret_cast<const float2*>(w.yi), p0,
+                                                                post.peaks);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
-  if ((e = launch_pdl(tc::tc_residual_kernel, D, 128, 0, stream, ev)) != cudaSuccess) return e;
+  if ((e = launch_pdl(tc::tc_residual_kernel, D, 128, 0, stream, ev, post.peaks)) != cudaSuccess) return e;
   if (prof && (e = cudaEventRecord(ctx->ev[3], stream)) != cudaSuccess) return e;
   return cudaSuccess;
 }

@@ -15,7 +15,8 @@
 // per (station, channel, j1) or (pair, polarisation, j1). Complex numbers are stored as
 // interleaved (re, im) pairs and the GEMMs are real: K = 1024, 256 output columns (forward)
 // and K = 256, 1024 output columns (inverse). The A-point DFTs over the sub-block phase and
-// the twiddles run in FP32 on the SIMT cores before (forward) and after (inverse) the GEMM.
+// the twiddles run in FP32 on the SIMT cores before (forward) and after (inverse) the GEMM, the
+// latter in its epilogue where that is possible (post_tile).
 //
 // Precision: the GEMMs run on tensor cores in BF16 with FP32 accumulation. Each FP32 operand
 // is split into BF16 parts (x = hi + mid + lo, each the round-to-nearest of what is left) and
@@ -119,6 +120,13 @@ struct GemmParams {
   unsigned* err;
   int ldd, chunks, chunks_per_group, terms;   // terms 3 or 6
   int m_tiles, n_tiles, groups;               // work items: (m tile, n tile, K group), n fastest
+  // the post-pass in the epilogue (see post_tile)
+  const float2* wn;            // [N] exp(-2 pi i x / N)
+  float* efield;               // [pairs][2][N] or null
+  float* envelope;             // [pairs][N] or null
+  unsigned long long* peaks;   // [pairs] see peak_word
+  long long pair0;             // the chunk's first pair
+  int n_pairs, k_lo;
 };
 
 // The work item of a persistent CTA's w-th item and the K chunks it covers.
@@ -186,6 +194,130 @@ __device__ __forceinline__ void tc_commit(uint64_t* bar) {
                : "memory");
 }
 
+// A pair's envelope peak as a word whose maximum over the pair's samples has the largest value and, on ties,
+// the lowest sample (values >= 0: their bits compare as integers); 0: none, all are NaN.
+__device__ __forceinline__ unsigned long long peak_word(float v, int n) {
+  return (static_cast<unsigned long long>(__float_as_uint(v)) << 32) | (0xffffffffu - static_cast<unsigned>(n));
+}
+
+// The post-pass in the GEMM's epilogue (tc_inverse_post_kernel: the same operations in the same order) on
+// 32 accumulator columns of a warp's 32 rows, which are 16 samples n2 of the A sub-blocks j1 of both
+// polarisations of 16 / A pairs. Lane i takes n2 = i % 16 of the pairs i / 16, i / 16 + 2, ...
+
+// the twiddles of sample n2: exp(-2 pi i j n2 / N) and exp(-2 pi i k_lo (n2 + 512 j) / N)
+template <int A>
+__device__ __forceinline__ void post_twiddles(const GemmParams& p, int n2, float2 (&tw)[A], float2 (&ph)[A]) {
+#pragma unroll
+  for (int j = 0; j < A; ++j) {
+    tw[j] = j == 0 ? make_float2(1.f, 0.f) : __ldg(p.wn + j * n2);
+    ph[j] = __ldg(p.wn + ((p.k_lo * (n2 + kSub * j)) & (A * kSub - 1)));
+  }
+}
+
+// x: row `lane` of the block; lp0: the warp's first pair in the chunk; n2: the lane's sample; buf: 2 KB of
+// shared memory of the warp, one polarisation's rows at a time (16-byte chunk j of row r at j ^ (r & 7): free
+// of bank conflicts); bv, bi: the running peaks.
+template <int A>
+__device__ __forceinline__ void post_block(const GemmParams& p, const uint32_t (&x)[32], int lane, int lp0, int n2,
+                                           const float2 (&tw)[A], const float2 (&ph)[A], float4* buf,
+                                           float (&bv)[8 / A], int (&bi)[8 / A]) {
+  constexpr int N = A * kSub, IT = 8 / A;   // pairs per lane
+  float pw[IT][A];
+#pragma unroll
+  for (int pol = 0; pol < 2; ++pol) {
+    // row (pair * 2 + pol) * A + j1 of the warp is row pair * A + j1 of the polarisation
+    if (((lane / A) & 1) == pol) {
+      const int r = (lane / (2 * A)) * A + lane % A;
+#pragma unroll
+      for (int j = 0; j < 8; ++j)
+        buf[r * 8 + (j ^ (r & 7))] = make_float4(__uint_as_float(x[4 * j]), __uint_as_float(x[4 * j + 1]),
+                                                 __uint_as_float(x[4 * j + 2]), __uint_as_float(x[4 * j + 3]));
+    }
+    __syncwarp();
+#pragma unroll
+    for (int it = 0; it < IT; ++it) {
+      const int pr = 2 * it + (lane >> 4), lp = lp0 + pr;
+      float2 y[A];
+#pragma unroll
+      for (int j1 = 0; j1 < A; ++j1) {
+        const int r = pr * A + j1, i = lane & 15;
+        const float2 v = reinterpret_cast<const float2*>(buf)[r * 16 + 2 * ((i >> 1) ^ (r & 7)) + (i & 1)];
+        y[j1] = j1 == 0 ? v : cmulc(v, tw[j1]);   // exp(+2 pi i j1 n2 / N)
+      }
+      dft<A, +1>(y);
+      const bool store = p.efield && lp < p.n_pairs;
+      float* ef = p.efield + (static_cast<size_t>(p.pair0 + lp) * 2 + pol) * N + n2;
+#pragma unroll
+      for (int n1 = 0; n1 < A; ++n1) {
+        const float2 zz = cmulc(y[n1], ph[n1]);   // exp(+2 pi i k_lo n / N)
+        if (store) ef[kSub * n1] = zz.x;
+        pw[it][n1] = pol == 0 ? cabs2(zz) : pw[it][n1] + cabs2(zz);
+      }
+    }
+    __syncwarp();   // the rows are read before the next ones overwrite them
+  }
+#pragma unroll
+  for (int it = 0; it < IT; ++it) {
+    const int lp = lp0 + 2 * it + (lane >> 4);
+    const bool store = p.envelope && lp < p.n_pairs;
+    float* en = p.envelope + static_cast<size_t>(p.pair0 + lp) * N + n2;
+#pragma unroll
+    for (int n1 = 0; n1 < A; ++n1) {
+      const float v = sqrtf(pw[it][n1]);
+      const int n = n2 + kSub * n1;   // not in order over the blocks of a tile
+      if (store) en[kSub * n1] = v;
+      if (v > bv[it] || (v == bv[it] && n < bi[it])) { bv[it] = v; bi[it] = n; }
+    }
+  }
+}
+
+// A finished tile's accumulator (at taddr, the warp's lanes): its blocks' outputs and the pairs' peaks. The next
+// block's twiddles (from L2: shared memory takes what L1 would need for them) are loaded a block ahead, with
+// two sub-blocks, where eight pairs per warp cover the latency, in place (43 x 29 pairs of 4096
+// samples 97.9 -> 94.4 us the call; 124 x 40 of 1024 86.1 ahead, 84.4 in place).
+template <int BN, int A>
+__device__ __forceinline__ void post_tile(const GemmParams& p, uint32_t taddr, int lane, int row0, int nt, float4* buf) {
+  constexpr bool kAhead = A > 2;
+  const int lp0 = row0 / (2 * A), n20 = nt * (BN / 2) + (lane & 15);
+  float bv[8 / A];
+  int bi[8 / A];
+#pragma unroll
+  for (int it = 0; it < 8 / A; ++it) {
+    bv[it] = -1.f;
+    bi[it] = 0;
+  }
+  float2 tw[A], ph[A];
+  if (kAhead) post_twiddles<A>(p, n20, tw, ph);
+#pragma unroll 1
+  for (int c = 0; c < BN; c += 32) {
+    uint32_t x[32];
+    tmem_ld32(taddr + c, x);
+    float2 tw_next[A], ph_next[A];
+    if (kAhead) post_twiddles<A>(p, n20 + ((c + 32) % BN) / 2, tw_next, ph_next);
+    else post_twiddles<A>(p, n20 + c / 2, tw, ph);
+    tmem_wait_ld();
+    post_block<A>(p, x, lane, lp0, n20 + c / 2, tw, ph, buf, bv, bi);
+    if (kAhead) {
+#pragma unroll
+      for (int j = 0; j < A; ++j) {
+        tw[j] = tw_next[j];
+        ph[j] = ph_next[j];
+      }
+    }
+  }
+#pragma unroll
+  for (int it = 0; it < 8 / A; ++it) {
+    unsigned long long best = bv[it] < 0.f ? 0ull : peak_word(bv[it], bi[it]);
+#pragma unroll
+    for (int off = 8; off > 0; off >>= 1) {
+      const unsigned long long o = __shfl_xor_sync(0xffffffffu, best, off);
+      if (o > best) best = o;
+    }
+    const int lp = lp0 + 2 * it + (lane >> 4);
+    if ((lane & 15) == 0 && best && lp < p.n_pairs) atomicMax(p.peaks + p.pair0 + lp, best);
+  }
+}
+
 // Accumulation. The tensor cores' FP32 accumulator loses about 2^-26 of relative precision,
 // with a bias, at every MMA (measured: the error grows linearly with the number of MMAs into
 // one accumulator), so each fold unit (up to eight 32-wide K chunks) is accumulated on its own
@@ -196,7 +328,14 @@ __device__ __forceinline__ void tc_commit(uint64_t* bar) {
 // are single fold units and need no S): P0, P1 of 256 columns.
 constexpr int kTmemCols = 512;
 
-template <int BN>
+//
+// A > 0: the inverse GEMM of traces of 512 A samples with the post-pass in place of the store of D, which
+// saves writing and reading it (82 MB each way for 43 x 29 pairs of 4096 samples: 119.3 -> 94.4 us the call,
+// 124 x 64 of 2048 265 -> 185). A tile holds every sub-block and both polarisations of its
+// pairs for a quarter of the samples n2; the peaks of a pair's tiles meet in p.peaks. Four warps run the epilogue beside
+// the next tile's MMAs; eight made the kernel 7 % faster (57 -> 53 us) but, with their registers, left the
+// SMs no room for the next call's first kernel (94.4 -> 101.7 us the call).
+template <int BN, int A = 0>
 __global__ void __launch_bounds__(kGemmThreads, 1) split_gemm_kernel(const __grid_constant__ GemmParams p) {
   static_assert(BN == 128 || BN == 256, "tile width");
   constexpr int NB = BN / 128;   // 128-row B blocks per tile
@@ -227,7 +366,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) split_gemm_kernel(const __gri
   // fold only moves the accumulator to global memory.
   const int F = cpg <= kFoldChunks ? cpg : cpg % 8 == 0 ? 8 : cpg % 4 == 0 ? 4 : cpg % 2 == 0 ? 2 : 1;
   const int nu = nk / F;   // fold units
-  if (NB == 2 && F != cpg) {   // the wide tile has no running sum
+  if ((NB == 2 || A > 0) && (F != cpg || (A > 0 && p.groups != 1))) {   // the wide tile has no running sum
     if (tid == 0) atomicOr(p.err, kErrBadLaunch);
     return;
   }
@@ -315,41 +454,46 @@ __global__ void __launch_bounds__(kGemmThreads, 1) split_gemm_kernel(const __gri
         drow = p.d + w.g * p.d_group + static_cast<size_t>(w.mt * kBM + 32 * warp) * p.ldd + w.nt * BN;
       }
       const uint32_t preg = t_sum + (NB == 2 ? BN * b : BN * (1 + b));
+      if constexpr (A > 0) {
+        const GemmItem w = gemm_item(p, i / cpg);
+        post_tile<BN, A>(p, preg + lanes, lane, w.mt * kBM + 32 * warp, w.nt, epi);
+      } else {
 #pragma unroll 1
-      for (int c = 0; c < BN; c += 32) {
-        uint32_t x[32], y[32];
-        tmem_ld32(preg + lanes + c, x);
-        if (!first) tmem_ld32(t_sum + lanes + c, y);
-        tmem_wait_ld();
-        if (!first) {
+        for (int c = 0; c < BN; c += 32) {
+          uint32_t x[32], y[32];
+          tmem_ld32(preg + lanes + c, x);
+          if (!first) tmem_ld32(t_sum + lanes + c, y);
+          tmem_wait_ld();
+          if (!first) {
 #pragma unroll
-          for (int k = 0; k < 32; ++k) x[k] = __float_as_uint(__fadd_rn(__uint_as_float(y[k]), __uint_as_float(x[k])));
-        }
-        if (last) {
-          // Lane l holds row l of the warp's 32 x 32 block. Transposed in two halves through shared
-          // memory (16-byte chunk j of row r at chunk j ^ ((r >> 1) & 3): both sides free of bank
-          // conflicts) so that each store instruction writes eight rows of 64 contiguous bytes.
-#pragma unroll
-          for (int hf = 0; hf < 2; ++hf) {
-#pragma unroll
-            for (int j = 0; j < 4; ++j)
-              epi[lane * 4 + (j ^ ((lane >> 1) & 3))] =
-                  make_float4(__uint_as_float(x[16 * hf + 4 * j]), __uint_as_float(x[16 * hf + 4 * j + 1]),
-                              __uint_as_float(x[16 * hf + 4 * j + 2]), __uint_as_float(x[16 * hf + 4 * j + 3]));
-            __syncwarp();
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-              const int r = 8 * i + (lane >> 2), ch = lane & 3;
-              *reinterpret_cast<float4*>(drow + static_cast<size_t>(r) * p.ldd + c + 16 * hf + 4 * ch) =
-                  epi[r * 4 + (ch ^ ((r >> 1) & 3))];
-            }
-            __syncwarp();   // the tile is read before the next half overwrites it
+            for (int k = 0; k < 32; ++k) x[k] = __float_as_uint(__fadd_rn(__uint_as_float(y[k]), __uint_as_float(x[k])));
           }
-        } else {
-          tmem_st32(t_sum + lanes + c, x);
+          if (last) {
+            // Lane l holds row l of the warp's 32 x 32 block. Transposed in two halves through shared
+            // memory (16-byte chunk j of row r at chunk j ^ ((r >> 1) & 3): both sides free of bank
+            // conflicts) so that each store instruction writes eight rows of 64 contiguous bytes.
+#pragma unroll
+            for (int hf = 0; hf < 2; ++hf) {
+#pragma unroll
+              for (int j = 0; j < 4; ++j)
+                epi[lane * 4 + (j ^ ((lane >> 1) & 3))] =
+                    make_float4(__uint_as_float(x[16 * hf + 4 * j]), __uint_as_float(x[16 * hf + 4 * j + 1]),
+                                __uint_as_float(x[16 * hf + 4 * j + 2]), __uint_as_float(x[16 * hf + 4 * j + 3]));
+              __syncwarp();
+#pragma unroll
+              for (int i = 0; i < 4; ++i) {
+                const int r = 8 * i + (lane >> 2), ch = lane & 3;
+                *reinterpret_cast<float4*>(drow + static_cast<size_t>(r) * p.ldd + c + 16 * hf + 4 * ch) =
+                    epi[r * 4 + (ch ^ ((r >> 1) & 3))];
+              }
+              __syncwarp();   // the tile is read before the next half overwrites it
+            }
+          } else {
+            tmem_st32(t_sum + lanes + c, x);
+          }
         }
+        if (!last) tmem_wait_st();
       }
-      if (!last) tmem_wait_st();
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(&pfree[b]);
@@ -436,7 +580,8 @@ template <int N_>
 __global__ void __launch_bounds__(kSolveThreads) tc_solve_kernel(const __grid_constant__ EventDesc ev,
                                                                  const float2* xf,
                                                                  const __grid_constant__ SplitImage img,
-                                                                 long long pair0, int n_pairs, int pairs_per_cta) {
+                                                                 long long pair0, int n_pairs, int pairs_per_cta,
+                                                                 unsigned long long* peaks) {
   constexpr int N = N_, M = N / 4, A = N / kSub, T = kSolveThreads;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   float4* hinv = reinterpret_cast<float4*>(smem_raw);                         // [2][M]
@@ -482,16 +627,20 @@ __global__ void __launch_bounds__(kSolveThreads) tc_solve_kernel(const __grid_co
       put_split(img.plane, img.planes, image_offset((lp * 2) * A + j1, 2 * j2, kInvK), et);
       put_split(img.plane, img.planes, image_offset((lp * 2 + 1) * A + j1, 2 * j2, kInvK), ep);
     }
-    if (tid == 0) ev.status[pair] = di.st | (key_sing ? kStSingular : 0u);
+    if (tid == 0) {
+      ev.status[pair] = di.st | (key_sing ? kStSingular : 0u);
+      if (peaks) peaks[pair] = 0ull;   // for the inverse GEMM, if that forms them
+    }
   }
 }
 
 // ---- inverse: twiddle, A-point DFT over the sub-block phase, band phase, envelope, peak ----
-// One CTA per pair of the chunk, thread n2; the inverse GEMM output holds Y[j1][n2] at row
-// ((lp * 2 + pol) * A + j1), complex column n2.
+// Where the GEMM's epilogue does not do it (post_block). One CTA per pair of the chunk, thread n2; the inverse
+// GEMM output holds Y[j1][n2] at row ((lp * 2 + pol) * A + j1), complex column n2.
 template <int N_>
 __global__ void __launch_bounds__(kSub) tc_inverse_post_kernel(const __grid_constant__ EventDesc ev,
-                                                               const float2* y_in, long long pair0) {
+                                                               const float2* y_in, long long pair0,
+                                                               unsigned long long* peaks) {
   constexpr int N = N_, A = N / kSub;
   const int lp = blockIdx.x, n2 = threadIdx.x;
   const long long pair = pair0 + lp;
@@ -544,6 +693,7 @@ __global__ void __launch_bounds__(kSub) tc_inverse_post_kernel(const __grid_cons
   if (n2 == 0) {
     for (int w = 1; w < kSub / 32; ++w)
       if (rv[w] > bv || (rv[w] == bv && ri[w] < bi)) { bv = rv[w]; bi = ri[w]; }
+    if (peaks) peaks[pair] = bv < 0.f ? 0ull : peak_word(bv, bi);   // an event whose other pairs' peaks are there
     if (bv < 0.f) { bv = 0.f; bi = 0; }
     pk_v = bv;
     pk_i = bi;
@@ -564,10 +714,20 @@ __global__ void __launch_bounds__(kSub) tc_inverse_post_kernel(const __grid_cons
 // ---- per direction: the FP64 plane-wave timing residual ------------------------------------
 // A kernel of its own: with a completion counter in the post-pass, whose CTA per pair lives only a few
 // microseconds, the release of every pair took that kernel from 29.5 to 43 us (1247 pairs at 4096).
-__global__ void __launch_bounds__(128) tc_residual_kernel(const __grid_constant__ EventDesc ev) {
+// peaks: the pairs' peak words from the inverse GEMM, or null (the post-pass has written the peaks).
+__global__ void __launch_bounds__(128) tc_residual_kernel(const __grid_constant__ EventDesc ev,
+                                                          const unsigned long long* peaks) {
   __shared__ double red[128 / 32];
   pdl_launch_dependents();
   pdl_wait_prior();
+  if (peaks) {   // each thread those that it reads below
+    for (int s = threadIdx.x; s < ev.n_st; s += 128) {
+      const size_t pair = static_cast<size_t>(blockIdx.x) * ev.n_st + s;
+      const unsigned long long w = __ldcg(peaks + pair);
+      ev.peak_idx[pair] = w ? static_cast<int>(0xffffffffu - static_cast<unsigned>(w)) : 0;
+      ev.peak_amp[pair] = __uint_as_float(static_cast<unsigned>(w >> 32));
+    }
+  }
   direction_residual<128>(ev, blockIdx.x, red);
 }
 
