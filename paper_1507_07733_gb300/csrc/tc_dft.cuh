@@ -510,12 +510,15 @@ __global__ void __launch_bounds__(kGemmThreads, 1) split_gemm_kernel(const __gri
 
 // Sum of the split-K groups' partial results, in group order (each group already folded its
 // chunks in order): out[i] = ((part[0][i] + part[1][i]) + ...).
+// Unrolled to the most groups (16), whose loads are then all in flight: a call of 10 x 10 pairs of 4096
+// samples 45.2 -> 43.3 us, 30 x 20 of 2048 43.95 -> 42.5.
 __global__ void tc_reduce_kernel(const float4* part, float4* out, size_t n4, size_t group4, int groups) {
   pdl_launch_dependents();
   pdl_wait_prior();
   for (size_t i = blockIdx.x * static_cast<size_t>(blockDim.x) + threadIdx.x; i < n4;
        i += static_cast<size_t>(gridDim.x) * blockDim.x) {
     float4 a = part[i];
+#pragma unroll 15
     for (int gi = 1; gi < groups; ++gi) {
       const float4 b = part[gi * group4 + i];
       a = make_float4(__fadd_rn(a.x, b.x), __fadd_rn(a.y, b.y), __fadd_rn(a.z, b.z), __fadd_rn(a.w, b.w));
