@@ -312,15 +312,15 @@ ar_status ensure_spec(ar_ctx* ctx, size_t bytes) {
   return AR_OK;
 }
 
-// the dynamic shared-memory limit of both unfold instantiations of a length
+// the dynamic shared-memory limit of the unfold instantiations of a length
 template <int N_>
 cudaError_t set_unfold_smem_limit(size_t bytes) {
-  cudaError_t e = cudaFuncSetAttribute(unfold_kernel<N_, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       static_cast<int>(bytes));
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(unfold_kernel<N_, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             static_cast<int>(bytes));
-  return e;
+  for (auto* kernel : {unfold_kernel<N_, false>, unfold_kernel<N_, true>, unfold_kernel<N_, false, true>}) {
+    const cudaError_t e =
+        cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(bytes));
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
 // The station kernel's shared memory, and its SMs' split between L1 and shared memory set for the
@@ -803,16 +803,18 @@ cudaError_t launch_recon(ar_ctx* ctx, const ar_event* ev, int max_iter, double t
   fp.tol_rad = tol_rad;
   fp.n_st = S;
   if ((e = launch_pdl(plane_fit_kernel, 1, 128, 0, stream, fp)) != cudaSuccess) return e;
+  // The unfold kernel's last CTA makes the iteration's fit; with SNRs a kernel of its own does.
+  const size_t smem = UnfoldSmem<N_>::total(pp.ev0.n_f_layout, pp.ev0.slab_direct != 0);
+  const int grid = std::min(rs.kc->grid, S);
+  fp.times = out->last.peak_time_ns;
+  fp.idx = out->last.peak_idx;
   for (int it = 1; it <= max_iter; ++it) {
-    const size_t smem = UnfoldSmem<N_>::total(pp.ev0.n_f_layout, pp.ev0.slab_direct != 0);
-    if ((e = pp.ev0.snr ? launch_pdl(unfold_kernel<N_, true>, std::min(rs.kc->grid, S), L::T, smem, stream, pp)
-                        : launch_pdl(unfold_kernel<N_, false>, std::min(rs.kc->grid, S), L::T, smem, stream, pp)) !=
-        cudaSuccess)
-      return e;
-    fp.times = out->last.peak_time_ns;
-    fp.idx = out->last.peak_idx;
     fp.iteration = it;
-    if ((e = launch_pdl(plane_fit_kernel, 1, 128, 0, stream, fp)) != cudaSuccess) return e;
+    pp.fit = fp;
+    if ((e = pp.ev0.snr ? launch_pdl(unfold_kernel<N_, true>, grid, L::T, smem, stream, pp)
+                        : launch_pdl(unfold_kernel<N_, false, true>, grid, L::T, smem, stream, pp)) != cudaSuccess ||
+        (pp.ev0.snr && (e = launch_pdl(plane_fit_kernel, 1, 128, 0, stream, fp)) != cudaSuccess))
+      return e;
   }
   return cudaSuccess;
 }

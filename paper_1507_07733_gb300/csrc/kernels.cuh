@@ -240,6 +240,33 @@ __host__ __device__ inline const EventDesc* batch_events(const BatchHeader* h) {
   return reinterpret_cast<const EventDesc*>(reinterpret_cast<const unsigned char*>(h) + 16);
 }
 
+// The iterative reconstruction (below): its state and what a plane-wave fit takes and gives.
+struct ReconState {        // device memory, one per ar_reconstruct call
+  double dir[2];           // direction the next unfold uses (zenith, azimuth)
+  double n[3];             // its unit vector
+  int converged;           // set when the direction stops changing (or the fit fails)
+  int pad;
+};
+
+struct FitParams {
+  const double* pos;       // [S][3]
+  const double* times;     // [S] station times to fit (voltage maxima, or the unfold's peak times)
+  const int* idx;          // [S] the sample indices behind those times
+  int* prev_idx;           // [S] the indices of the previous fit (updated here)
+  ReconState* st;
+  DirPre* dir_pre;         // the direction's cell and vector for the next unfold kernel
+  PatternRef pattern;      // the event's own pattern
+  int own_pattern;         // 0: stations have patterns of their own, no cell is formed
+  // the results of the last fit made: the caller's outputs, written by every fit
+  double* direction;       // [2]
+  double* t0;
+  double* chi2;
+  int* iterations;
+  double* history;         // [(max_iter + 1)][2] or null
+  double n_over_c, tol_rad;
+  int n_st, iteration;     // iteration 0 fits the voltage maxima
+};
+
 struct PathParams {
   const BatchHeader* batch;   // device batch, or null: the single event ev0
   unsigned* err;              // device error word
@@ -253,6 +280,7 @@ struct PathParams {
   // The copies themselves are unchanged and in bounds. 0 in every other launch.
   int test_wait;
   EventDesc ev0;
+  FitParams fit;              // (unfold kernel of an iteration) the fit that its last CTA makes
 };
 
 // a / b and a mod b of a count a >= 0 (a 64-bit division takes several times a 32-bit one)
@@ -1000,9 +1028,185 @@ __device__ __forceinline__ bool build_inverse(const EventDesc& ev, int p, const 
   return __syncthreads_or(sing);
 }
 
+// The 12 values v of each lane summed over the warp: the result of value i lies in the lanes of
+// slot i (warp_sum12_slot). Half of the values go to the other half of the lanes at each step, 13
+// additions where a butterfly per value takes 60 (an FP64 instruction occupies an SM's two FP64 lanes for
+// 16 cycles). The order is fixed.
+__device__ __forceinline__ int warp_sum12_slot(int lane) {   // -1: none
+  const int low = ((lane >> 2) & 1) * 2 + ((lane >> 1) & 1);
+  return low < 3 ? (lane >> 4) * 6 + ((lane >> 3) & 1) * 3 + low : -1;
+}
+__device__ __forceinline__ double warp_sum12(double (&v)[12], int lane) {
+  const auto step = [&](auto half, int off) {
+    constexpr int H = decltype(half)::value;
+    const bool up = (lane & off) != 0;
+#pragma unroll
+    for (int i = 0; i < H; ++i) {
+      const double give = up ? v[i] : v[i + H], keep = up ? v[i + H] : v[i];
+      v[i] = keep + __shfl_xor_sync(0xffffffffu, give, off);
+    }
+  };
+  step(std::integral_constant<int, 6>{}, 16);
+  step(std::integral_constant<int, 3>{}, 8);
+  v[3] = 0.0;
+  step(std::integral_constant<int, 2>{}, 4);
+  step(std::integral_constant<int, 1>{}, 2);
+  return v[0] + __shfl_xor_sync(0xffffffffu, v[0], 1);
+}
+
+// Least-squares plane wave t_s = t0 - n.x_s n_refr / c: linear in (t0, nx, ny) for a fixed nz,
+// repeated four times with nz from the previous solution (nz = 1 first). 128 threads of a
+// CTA of T, FP64, sums in a fixed order. Also decides convergence and the residual chi2.
+//
+// FP64 runs at 1/64 of the FP32 rate here, so a fit is bound by its FP64 instructions and their
+// chains, and does each thing once: the station sums once for all four repetitions (the right-hand
+// side t + k nz z is linear in nz, so the solution is a + nz b), the matrix inverted once by its
+// cofactors, one thread's scalars for the repetitions, the mean residual from the sums, and the two
+// arc tangents, the convergence test and the next unfold's pattern cell on lanes of different
+// warps side by side. 124 stations: 44 us with sums per repetition and every thread repeating the
+// trigonometry, 12.0 us now (ncu, one launch at a time). The unfold kernel of an iteration ends with the
+// fit: a kernel for each fit made 19 launches of a reconstruction of 8 iterations, now 11 (98 -> 85 us).
+template <int T>
+__device__ __forceinline__ void plane_fit(const FitParams& p) {
+  ReconState* st = p.st;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  __shared__ double red[4][12];
+  __shared__ double tot[12];
+  __shared__ double sol[6];       // t0, nx, ny, nz, mean residual time, horizontal component
+  __shared__ double angle[2];     // zenith, azimuth
+  __shared__ double pos[2];       // their positions in the pattern's table
+  __shared__ int flags[4];        // [0] a direction was found, [1] converged, [2], [3] of the positions
+  const double k = p.n_over_c;
+  // do the station indices repeat those of the previous fit?
+  int diff = 0;
+  double v[12] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0};   // x, y, xx, xy, yy, t, xt, yt, z, xz, yz
+  for (int s = tid; tid < 128 && s < p.n_st; s += 128) {
+    const double x = p.pos[3 * s], y = p.pos[3 * s + 1], z = p.pos[3 * s + 2], t = __ldcg(p.times + s);
+    v[0] += x; v[1] += y; v[2] += x * x; v[3] += x * y; v[4] += y * y;
+    v[5] += t; v[6] += x * t; v[7] += y * t;
+    v[8] += z; v[9] += x * z; v[10] += y * z;
+    const int i = __ldcg(p.idx + s);
+    diff |= p.iteration > 0 && i != p.prev_idx[s];
+    p.prev_idx[s] = i;
+  }
+  const double total = warp_sum12(v, lane);
+  const int slot = warp_sum12_slot(lane);
+  if (slot >= 0 && (lane & 1) == 0 && warp < 4) red[warp][slot] = total;
+  const int same = !__syncthreads_or(diff) && p.iteration > 0;
+  if (warp == 0) {
+    if (lane < 12) tot[lane] = red[0][lane] + red[1][lane] + red[2][lane] + red[3][lane];
+    __syncwarp();
+    if (lane == 0) {
+      const double n = p.n_st, sx = tot[0], sy = tot[1], sxx = tot[2], sxy = tot[3], syy = tot[4];
+      const double c00 = sxx * syy - sxy * sxy, c01 = sxy * sy - sx * syy, c02 = sx * sxy - sxx * sy;
+      const double c11 = n * syy - sy * sy, c12 = sx * sy - n * sxy, c22 = n * sxx - sx * sx;
+      const double det = n * c00 + sx * c01 + sy * c02;
+      const bool ok = fabs(det) > 1e-12 * (n * sxx * syy);
+      flags[0] = ok ? 1 : 0;
+      if (ok) {
+        const double inv = 1.0 / det, inv_k = 1.0 / (k * det);
+        // the solution of the right-hand sides t and k z: t0 and -(nx, ny) k
+        const double a0 = (c00 * tot[5] + c01 * tot[6] + c02 * tot[7]) * inv;
+        const double a1 = -(c01 * tot[5] + c11 * tot[6] + c12 * tot[7]) * inv_k;
+        const double a2 = -(c02 * tot[5] + c12 * tot[6] + c22 * tot[7]) * inv_k;
+        const double b0 = k * (c00 * tot[8] + c01 * tot[9] + c02 * tot[10]) * inv;
+        const double b1 = -(c01 * tot[8] + c11 * tot[9] + c12 * tot[10]) * inv;
+        const double b2 = -(c02 * tot[8] + c12 * tot[9] + c22 * tot[10]) * inv;
+        double nx = 0.0, ny = 0.0, nz = 1.0, t0 = 0.0, h2 = 0.0;
+        for (int pass = 0; pass < 4; ++pass) {
+          t0 = a0 + nz * b0;
+          nx = a1 + nz * b1;
+          ny = a2 + nz * b2;
+          h2 = nx * nx + ny * ny;
+          if (h2 > 1.0) {
+            const double h = sqrt(h2);
+            nx /= h;
+            ny /= h;
+            h2 = 1.0;
+          }
+          nz = sqrt(1.0 - h2);
+        }
+        sol[0] = t0;
+        sol[1] = nx;
+        sol[2] = ny;
+        sol[3] = nz;
+        sol[4] = (tot[5] + k * (nx * sx + ny * sy + nz * tot[8])) / n;
+        sol[5] = h2;
+      }
+    }
+  }
+  __syncthreads();
+  if (!flags[0]) {   // no direction: stop; the first fit failing marks the reconstruction failed
+    if (tid == 0) {
+      st->converged = 1;
+      if (p.iteration == 0) p.direction[0] = p.direction[1] = *p.t0 = *p.chi2 = __longlong_as_double(0x7ff8000000000000ll);
+      *p.iterations = p.iteration == 0 ? -1 : p.iteration;
+    }
+    return;
+  }
+  const double nx = sol[1], ny = sol[2], nz = sol[3], mean = sol[4];
+  // chi2 of this direction with these times
+  double ss = 0.0;
+  for (int s = tid; tid < 128 && s < p.n_st; s += 128) {
+    const double r = __ldcg(p.times + s) + (nx * p.pos[3 * s] + ny * p.pos[3 * s + 1] + nz * p.pos[3 * s + 2]) * k - mean;
+    ss += r * r;
+  }
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, off);
+  if (lane == 0 && warp < 4) {
+    red[warp][0] = ss;
+    if (warp == 1) {
+      angle[0] = atan2(sqrt(sol[5]), nz);
+      bool clamped;
+      flags[2] = zenith_position(p.pattern, angle[0], &pos[0], &clamped) ? (clamped ? 2 : 1) : 0;
+    } else if (warp == 2) {
+      double az = atan2(ny, nx);
+      if (az < 0.0) az += 2.0 * 3.14159265358979323846;
+      angle[1] = az;
+      flags[3] = azimuth_position(p.pattern, az, &pos[1]) ? 1 : 0;
+    } else if (warp == 3) {
+      bool done = false;
+      if (p.iteration > 0) {
+        double dot = st->n[0] * nx + st->n[1] * ny + st->n[2] * nz;
+        dot = dot > 1.0 ? 1.0 : (dot < -1.0 ? -1.0 : dot);
+        done = same || acos(dot) < p.tol_rad;
+      }
+      flags[1] = done ? 1 : 0;
+    }
+  }
+  __syncthreads();
+  if (tid == 0) {
+    const double zen = angle[0], az = angle[1];
+    st->dir[0] = zen;
+    st->dir[1] = az;
+    st->n[0] = nx;
+    st->n[1] = ny;
+    st->n[2] = nz;
+    if (flags[1]) st->converged = 1;
+    DirPre* dp = p.dir_pre;
+    dp->cell = p.own_pattern ? cell_of_positions(p.pattern, flags[2] && flags[3], pos[0], flags[2] == 2, pos[1]) : DirInfo{};
+    dp->n[0] = nx;
+    dp->n[1] = ny;
+    dp->n[2] = nz;
+    dp->pad = 0.0;
+  } else if (tid == 32) {
+    p.direction[0] = angle[0];
+    p.direction[1] = angle[1];
+    *p.t0 = sol[0];
+    *p.chi2 = red[0][0] + red[1][0] + red[2][0] + red[3][0];
+    *p.iterations = p.iteration;
+    if (p.history) {
+      p.history[2 * p.iteration] = angle[0];
+      p.history[2 * p.iteration + 1] = angle[1];
+    }
+  }
+}
+
 // kSnr: the instantiation that can compute pulse SNRs (for events that request them); the
 // other one carries none of that code, which costs the plain path time even when unused.
-template <int N_, bool kSnr>
+// kFit: the instantiation of an iteration of the reconstruction, whose last CTA also fits the plane wave
+// to the peaks: the next iteration's direction, or the end of the loop.
+template <int N_, bool kSnr, bool kFit = false>
 __global__ void __launch_bounds__(Layout<N_>::T, Layout<N_>::MIN_CTAS) unfold_kernel(const __grid_constant__ PathParams prm) {
   using L = Layout<N_>;
   using SM = UnfoldSmem<N_>;
@@ -1070,8 +1274,11 @@ __global__ void __launch_bounds__(Layout<N_>::T, Layout<N_>::MIN_CTAS) unfold_ke
   const bool early =
       static_cast<int>(blockIdx.x) < prm.n_early && prm.skip == nullptr && evs[e0].st_walk == nullptr;
   if (!early) {
+    // A loop's kernels all wait for the one before them, so the next one's launch need not wait for this
+    // wait (the launches left after convergence follow one another sooner).
+    if (prm.skip) pdl_launch_dependents();
     if (prm.wait_prior) pdl_wait_prior();
-    pdl_launch_dependents();
+    if (!prm.skip) pdl_launch_dependents();
     if (prm.skip && *prm.skip) return;
   }
   int s, p;
@@ -1378,6 +1585,12 @@ __global__ void __launch_bounds__(Layout<N_>::T, Layout<N_>::MIN_CTAS) unfold_ke
       pairs_in_dir = 0;
       __syncthreads();
       if (*sflag) direction_residual<T>(ev, d, redd);
+      if constexpr (kFit) {
+        if (*sflag) {
+          __syncthreads();   // the peak times are written
+          plane_fit<T>(prm.fit);
+        }
+      }
     }
     if (!has_next) break;
     __syncthreads();   // A, reductions and the event copy free for the next pair
@@ -1392,32 +1605,6 @@ __global__ void __launch_bounds__(Layout<N_>::T, Layout<N_>::MIN_CTAS) unfold_ke
 }
 
 // ---- iterative reconstruction (Sec. 2): voltage-maximum timing, plane-wave fit -------------
-
-struct ReconState {        // device memory, one per ar_reconstruct call
-  double dir[2];           // direction the next unfold uses (zenith, azimuth)
-  double n[3];             // its unit vector
-  int converged;           // set when the direction stops changing (or the fit fails)
-  int pad;
-};
-
-struct FitParams {
-  const double* pos;       // [S][3]
-  const double* times;     // [S] station times to fit (voltage maxima, or the unfold's peak times)
-  const int* idx;          // [S] the sample indices behind those times
-  int* prev_idx;           // [S] the indices of the previous fit (updated here)
-  ReconState* st;
-  DirPre* dir_pre;         // the direction's cell and vector for the next unfold kernel
-  PatternRef pattern;      // the event's own pattern
-  int own_pattern;         // 0: stations have patterns of their own, no cell is formed
-  // the results of the last fit made: the caller's outputs, written by every fit
-  double* direction;       // [2]
-  double* t0;
-  double* chi2;
-  int* iterations;
-  double* history;         // [(max_iter + 1)][2] or null
-  double n_over_c, tol_rad;
-  int n_st, iteration;     // iteration 0 fits the voltage maxima
-};
 
 // argmax_n v0[n]^2 + v1[n]^2 per station (FP64 squares, lowest index on ties); one CTA per station.
 // The first CTA also readies the loop's state and history (n_history doubles, or null). Runs
@@ -1435,10 +1622,27 @@ __global__ void __launch_bounds__(256) voltage_peak_kernel(const float* traces, 
   }
   const float* v0 = traces + static_cast<size_t>(s) * 2 * n;
   const float* v1 = v0 + n;
+  // The largest of the FP32 sums of squares, each within 2^-22 of its FP64 sum where neither over- nor
+  // underflows, leaves few samples whose FP64 sum can be the largest (all of them in FP64, six slow
+  // operations each: 9.2 us for 124 stations of 2048 samples; a reconstruction 85 -> 80 us with the earlier
+  // launches of its iterations).
+  float top = -1.f;
+  for (int j = tid; j < n; j += 256) top = fmaxf(top, fmaf(v0[j], v0[j], v1[j] * v1[j]));
+  __shared__ int stop;
+  if (tid == 0) stop = __float_as_int(-1.f);
+  __syncthreads();
+  // (values >= 0, or -1: their bits compare as integers)
+  const int wtop = __reduce_max_sync(0xffffffffu, __float_as_int(top));
+  if ((tid & 31) == 0) atomicMax(&stop, wtop);
+  __syncthreads();
+  top = __int_as_float(stop);
+  const float floor32 = top > 1e-30f && top < 1e38f ? top * (1.f - 0x1p-20f) : -1.f;
   double bv = -1.0;
   int bi = 0;
   for (int j = tid; j < n; j += 256) {
-    const double a = v0[j], b = v1[j];
+    const float a32 = v0[j], b32 = v1[j];
+    if (fmaf(a32, a32, b32 * b32) < floor32) continue;
+    const double a = a32, b = b32;
     const double pw = __dadd_rn(__dmul_rn(a, a), __dmul_rn(b, b));
     if (pw > bv) { bv = pw; bi = j; }
   }
@@ -1461,180 +1665,12 @@ __global__ void __launch_bounds__(256) voltage_peak_kernel(const float* traces, 
   pdl_wait_prior();
 }
 
-// The 12 values v of each lane summed over the warp: the result of value i lies in the lanes of
-// slot i (warp_sum12_slot). Half of the values go to the other half of the lanes at each step, 13
-// additions where a butterfly per value takes 60 (an FP64 instruction occupies an SM's two FP64 lanes for
-// 16 cycles). The order is fixed.
-__device__ __forceinline__ int warp_sum12_slot(int lane) {   // -1: none
-  const int low = ((lane >> 2) & 1) * 2 + ((lane >> 1) & 1);
-  return low < 3 ? (lane >> 4) * 6 + ((lane >> 3) & 1) * 3 + low : -1;
-}
-__device__ __forceinline__ double warp_sum12(double (&v)[12], int lane) {
-  const auto step = [&](auto half, int off) {
-    constexpr int H = decltype(half)::value;
-    const bool up = (lane & off) != 0;
-#pragma unroll
-    for (int i = 0; i < H; ++i) {
-      const double give = up ? v[i] : v[i + H], keep = up ? v[i + H] : v[i];
-      v[i] = keep + __shfl_xor_sync(0xffffffffu, give, off);
-    }
-  };
-  step(std::integral_constant<int, 6>{}, 16);
-  step(std::integral_constant<int, 3>{}, 8);
-  v[3] = 0.0;
-  step(std::integral_constant<int, 2>{}, 4);
-  step(std::integral_constant<int, 1>{}, 2);
-  return v[0] + __shfl_xor_sync(0xffffffffu, v[0], 1);
-}
-
-// Least-squares plane wave t_s = t0 - n.x_s n_refr / c: linear in (t0, nx, ny) for a fixed nz,
-// repeated four times with nz from the previous solution (nz = 1 first). One CTA of 128
-// threads, FP64, sums in a fixed order. Also decides convergence and the residual chi2.
-//
-// FP64 runs at 1/64 of the FP32 rate here, so the kernel is bound by its FP64 instructions and their
-// chains, and does each thing once: the station sums once for all four repetitions (the right-hand
-// side t + k nz z is linear in nz, so the solution is a + nz b), the matrix inverted once by its
-// cofactors, one thread's scalars for the repetitions, the mean residual from the sums, and the two
-// arc tangents, the convergence test and the next unfold's pattern cell on lanes of different
-// warps side by side. 124 stations: 44 us with sums per repetition and every thread repeating the
-// trigonometry, 12.7 us now (ncu, one launch at a time); the unfold kernel that takes the cell and
-// the source vector from here 19.5 -> 15.2 us.
+// The first fit, of the voltage maxima (the others are made by the unfold kernel).
 __global__ void __launch_bounds__(128) plane_fit_kernel(const __grid_constant__ FitParams p) {
   pdl_launch_dependents();
   pdl_wait_prior();
-  ReconState* st = p.st;
-  if (st->converged) return;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  __shared__ double red[4][12];
-  __shared__ double tot[12];
-  __shared__ double sol[6];       // t0, nx, ny, nz, mean residual time, horizontal component
-  __shared__ double angle[2];     // zenith, azimuth
-  __shared__ double pos[2];       // their positions in the pattern's table
-  __shared__ int flags[4];        // [0] a direction was found, [1] converged, [2], [3] of the positions
-  const double k = p.n_over_c;
-  // do the station indices repeat those of the previous fit?
-  int diff = 0;
-  double v[12] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0};   // x, y, xx, xy, yy, t, xt, yt, z, xz, yz
-  for (int s = tid; s < p.n_st; s += 128) {
-    const double x = p.pos[3 * s], y = p.pos[3 * s + 1], z = p.pos[3 * s + 2], t = p.times[s];
-    v[0] += x; v[1] += y; v[2] += x * x; v[3] += x * y; v[4] += y * y;
-    v[5] += t; v[6] += x * t; v[7] += y * t;
-    v[8] += z; v[9] += x * z; v[10] += y * z;
-    const int i = p.idx[s];
-    diff |= p.iteration > 0 && i != p.prev_idx[s];
-    p.prev_idx[s] = i;
-  }
-  const double total = warp_sum12(v, lane);
-  const int slot = warp_sum12_slot(lane);
-  if (slot >= 0 && (lane & 1) == 0) red[warp][slot] = total;
-  const int same = !__syncthreads_or(diff) && p.iteration > 0;
-  if (warp == 0) {
-    if (lane < 12) tot[lane] = red[0][lane] + red[1][lane] + red[2][lane] + red[3][lane];
-    __syncwarp();
-    if (lane == 0) {
-      const double n = p.n_st, sx = tot[0], sy = tot[1], sxx = tot[2], sxy = tot[3], syy = tot[4];
-      const double c00 = sxx * syy - sxy * sxy, c01 = sxy * sy - sx * syy, c02 = sx * sxy - sxx * sy;
-      const double c11 = n * syy - sy * sy, c12 = sx * sy - n * sxy, c22 = n * sxx - sx * sx;
-      const double det = n * c00 + sx * c01 + sy * c02;
-      const bool ok = fabs(det) > 1e-12 * (n * sxx * syy);
-      flags[0] = ok ? 1 : 0;
-      if (ok) {
-        const double inv = 1.0 / det, inv_k = 1.0 / (k * det);
-        // the solution of the right-hand sides t and k z: t0 and -(nx, ny) k
-        const double a0 = (c00 * tot[5] + c01 * tot[6] + c02 * tot[7]) * inv;
-        const double a1 = -(c01 * tot[5] + c11 * tot[6] + c12 * tot[7]) * inv_k;
-        const double a2 = -(c02 * tot[5] + c12 * tot[6] + c22 * tot[7]) * inv_k;
-        const double b0 = k * (c00 * tot[8] + c01 * tot[9] + c02 * tot[10]) * inv;
-        const double b1 = -(c01 * tot[8] + c11 * tot[9] + c12 * tot[10]) * inv;
-        const double b2 = -(c02 * tot[8] + c12 * tot[9] + c22 * tot[10]) * inv;
-        double nx = 0.0, ny = 0.0, nz = 1.0, t0 = 0.0, h2 = 0.0;
-        for (int pass = 0; pass < 4; ++pass) {
-          t0 = a0 + nz * b0;
-          nx = a1 + nz * b1;
-          ny = a2 + nz * b2;
-          h2 = nx * nx + ny * ny;
-          if (h2 > 1.0) {
-            const double h = sqrt(h2);
-            nx /= h;
-            ny /= h;
-            h2 = 1.0;
-          }
-          nz = sqrt(1.0 - h2);
-        }
-        sol[0] = t0;
-        sol[1] = nx;
-        sol[2] = ny;
-        sol[3] = nz;
-        sol[4] = (tot[5] + k * (nx * sx + ny * sy + nz * tot[8])) / n;
-        sol[5] = h2;
-      }
-    }
-  }
-  __syncthreads();
-  if (!flags[0]) {   // no direction: stop; the first fit failing marks the reconstruction failed
-    if (tid == 0) {
-      st->converged = 1;
-      if (p.iteration == 0) p.direction[0] = p.direction[1] = *p.t0 = *p.chi2 = __longlong_as_double(0x7ff8000000000000ll);
-      *p.iterations = p.iteration == 0 ? -1 : p.iteration;
-    }
-    return;
-  }
-  const double nx = sol[1], ny = sol[2], nz = sol[3], mean = sol[4];
-  // chi2 of this direction with these times
-  double ss = 0.0;
-  for (int s = tid; s < p.n_st; s += 128) {
-    const double r = p.times[s] + (nx * p.pos[3 * s] + ny * p.pos[3 * s + 1] + nz * p.pos[3 * s + 2]) * k - mean;
-    ss += r * r;
-  }
-#pragma unroll
-  for (int off = 16; off > 0; off >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, off);
-  if (lane == 0) {
-    red[warp][0] = ss;
-    if (warp == 1) {
-      angle[0] = atan2(sqrt(sol[5]), nz);
-      bool clamped;
-      flags[2] = zenith_position(p.pattern, angle[0], &pos[0], &clamped) ? (clamped ? 2 : 1) : 0;
-    } else if (warp == 2) {
-      double az = atan2(ny, nx);
-      if (az < 0.0) az += 2.0 * 3.14159265358979323846;
-      angle[1] = az;
-      flags[3] = azimuth_position(p.pattern, az, &pos[1]) ? 1 : 0;
-    } else if (warp == 3) {
-      bool done = false;
-      if (p.iteration > 0) {
-        double dot = st->n[0] * nx + st->n[1] * ny + st->n[2] * nz;
-        dot = dot > 1.0 ? 1.0 : (dot < -1.0 ? -1.0 : dot);
-        done = same || acos(dot) < p.tol_rad;
-      }
-      flags[1] = done ? 1 : 0;
-    }
-  }
-  __syncthreads();
-  if (tid == 0) {
-    const double zen = angle[0], az = angle[1];
-    st->dir[0] = zen;
-    st->dir[1] = az;
-    st->n[0] = nx;
-    st->n[1] = ny;
-    st->n[2] = nz;
-    if (flags[1]) st->converged = 1;
-    DirPre* dp = p.dir_pre;
-    dp->cell = p.own_pattern ? cell_of_positions(p.pattern, flags[2] && flags[3], pos[0], flags[2] == 2, pos[1]) : DirInfo{};
-    dp->n[0] = nx;
-    dp->n[1] = ny;
-    dp->n[2] = nz;
-    dp->pad = 0.0;
-  } else if (tid == 32) {
-    p.direction[0] = angle[0];
-    p.direction[1] = angle[1];
-    *p.t0 = sol[0];
-    *p.chi2 = red[0][0] + red[1][0] + red[2][0] + red[3][0];
-    *p.iterations = p.iteration;
-    if (p.history) {
-      p.history[2 * p.iteration] = angle[0];
-      p.history[2 * p.iteration + 1] = angle[1];
-    }
-  }
+  if (p.st->converged) return;
+  plane_fit<128>(p);
 }
 
 }  // namespace aerafold
