@@ -758,8 +758,8 @@ def run_output_variant(binding, synth, ctx, pid, dev, stream, hbm=None, variant=
 
 def run_tensor_core(binding, synth, ctx, pid, dev, stream, peaks, reps=20):
     """Throughput of the tensor-core variant on the scan workload (124 stations x 64
-    directions x 2048 samples): unfolds/s per call, and the inverse GEMM's tensor rate
-    (split products counted: 2 x rows x K x 1024 x terms, rows = 2 x pairs x 4) against the
+    directions x 2048 samples): unfolds/s per call, and the tensor rate of the inverse GEMM, whose
+    time includes the post-pass in its epilogue (split products counted: 2 x rows x K x 1024 x terms, rows = 2 x pairs x 4) against the
     measured dense BF16 peak."""
     import torch
     ev = synth.direction_scan()

@@ -247,8 +247,9 @@ ar_status ar_kernel_times(ar_ctx* ctx, float* ms);
  * 2^25 / N pairs).
  * ev, out: as ar_unfold (device memory); S * N <= 2^24.
  * With ar_set_profiling on, ar_kernel_times gives ms[0] = forward transform and the first
- * chunk's solve, ms[1] = the first chunk's inverse GEMM, ms[2] = the rest (post-pass, later
- * chunks, residual).
+ * chunk's solve, ms[1] = the first chunk's inverse GEMM (with the post-pass, unless sub-sample times,
+ * SNRs or few pairs leave that to a kernel of its own), ms[2] = the rest (that kernel, later chunks,
+ * residual).
  * Errors: as ar_unfold, and AR_ERR_INVALID_ARG for split_terms not 3 or 6 or S * N > 2^24. */
 ar_status ar_unfold_tc(ar_ctx* ctx, const ar_event* ev, const ar_outputs* out, int32_t split_terms, void* stream);
 
