@@ -1338,6 +1338,9 @@ __global__ void __launch_bounds__(Layout<N_>::T, Layout<N_>::MIN_CTAS) unfold_ke
             mbar_wait_bounded(bar, phase, limit);
           }
           if (copies_out) tma_bulk_wait_all();
+          // An early CTA has not waited for the station kernel yet, and the next call's first kernel waits for
+          // this grid alone: it would overwrite the spectra of a station kernel still running.
+          if (prm.wait_prior) pdl_wait_prior();
           __syncthreads();
           return;
         }

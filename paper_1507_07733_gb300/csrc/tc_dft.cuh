@@ -368,6 +368,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) split_gemm_kernel(const __gri
   const int nu = nk / F;   // fold units
   if ((NB == 2 || A > 0) && (F != cpg || (A > 0 && p.groups != 1))) {   // the wide tile has no running sum
     if (tid == 0) atomicOr(p.err, kErrBadLaunch);
+    pdl_wait_prior();   // the kernels behind rely on this one's end for everything before it
     return;
   }
 
