@@ -1015,6 +1015,17 @@ uint16_t bf16_bits(double x, double* value) {
   return static_cast<uint16_t>(u >> 16);
 }
 
+// Dynamic shared memory of the solve: per-bin inverses [2][N/4] float4, then the node scratch [n_f][8] float2
+template <int N_>
+size_t tc_solve_smem(int n_f) {
+  return 2 * sizeof(float4) * (N_ / 4) + sizeof(float2) * 8 * static_cast<size_t>(n_f);
+}
+template <int N_>
+cudaError_t tc_solve_limit() {
+  return cudaFuncSetAttribute(tc::tc_solve_kernel<N_>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              static_cast<int>(tc_solve_smem<N_>(kMaxFreqNodes)));
+}
+
 // The two real DFT matrices of the four-step transforms, split into three BF16 planes from
 // FP64 and laid out as the GEMM's shared-memory image. Rows are output columns, columns the
 // K index; complex values are interleaved (re, im).
@@ -1051,6 +1062,10 @@ ar_status build_tc_tables(ar_ctx* ctx) {
       AR_CUDA(ctx, cudaMemcpy(ctx->tc_b[which][pl], img[pl].data(), bytes, cudaMemcpyHostToDevice));
     }
   }
+  // (the largest patterns' node scratch takes the solve at 4096 samples past the default 48 KB)
+  AR_CUDA(ctx, tc_solve_limit<1024>());
+  AR_CUDA(ctx, tc_solve_limit<2048>());
+  AR_CUDA(ctx, tc_solve_limit<4096>());
   for (auto* kernel : {tc::split_gemm_kernel<128>, tc::split_gemm_kernel<256>, tc::split_gemm_kernel<256, 2>,
                        tc::split_gemm_kernel<256, 4>, tc::split_gemm_kernel<256, 8>})
     AR_CUDA(ctx, cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -1168,8 +1183,7 @@ cudaError_t launch_tc(ar_ctx* ctx, const EventDesc& ev, int terms, size_t rows_f
                       0, stream, ev, fimg)) != cudaSuccess)
     return e;
   if ((e = launch_gemm(ctx, w.fa, rows_f, 0, terms, w.xf, w.part, stream)) != cudaSuccess) return e;
-  // per-bin inverses [2][N/4] float4, then the node scratch [n_f][8] float2
-  const size_t solve_smem = 2 * sizeof(float4) * (N_ / 4) + sizeof(float2) * 8 * static_cast<size_t>(ev.n_f_layout);
+  const size_t solve_smem = tc_solve_smem<N_>(ev.n_f_layout);
   int solve_per_sm = 0;
   if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&solve_per_sm, tc::tc_solve_kernel<N_>, tc::kSolveThreads,
                                                          solve_smem)) != cudaSuccess)

@@ -173,3 +173,16 @@ def test_fine_times_and_snr_on_the_scan(env):
     assert np.all(abs(tc["snr"][same] - fp["snr"][same]) <= 1e-4 * fp["snr"][same])
     e = rel_l2(tc["envelope"], fp["envelope"], ev.n_samples)
     assert e.max() <= 1e-5, e.max()
+
+
+@pytest.mark.parametrize("n", [1024, 2048, 4096])
+def test_x6_parity_at_the_most_frequency_nodes(n):
+    """256 nodes, the most a pattern may have: the solve's largest shared memory (at 4096 samples past 48 KB)."""
+    from paper_1507_07733_gb300 import binding
+    grid = dict(synth.PATTERN_GRID, n_zen=7, dzen_deg=15.0, n_az=24, daz_deg=15.0, n_freq=256, df_hz=50e6 / 255)
+    pat = synth.make_pattern(seed_key=256, grid=grid)
+    ctx = binding.Context(0)
+    pid = ctx.load_pattern(pat)
+    ev = synth.make_event(9, n, synth.random_directions(3, np.random.default_rng(n)), seed_key=980 + n)
+    check_event(_run(ctx, pid, ev, 6), oracle.unfold_event(pat, ev), ev)
+    ctx.close()
