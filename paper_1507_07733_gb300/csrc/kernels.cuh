@@ -1068,6 +1068,7 @@ __device__ __forceinline__ double warp_sum12(double (&v)[12], int lane) {
 // fit: a kernel for each fit made 19 launches of a reconstruction of 8 iterations, now 11 (98 -> 85 us).
 template <int T>
 __device__ __forceinline__ void plane_fit(const FitParams& p) {
+  static_assert(T >= 128, "four warps: the sums' partials, the angles and the convergence test");
   ReconState* st = p.st;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   __shared__ double red[4][12];
