@@ -412,6 +412,9 @@ __global__ void __launch_bounds__(SpectrumSmem<N_>::BLOCK, 4) station_spectrum_k
   float2* x1 = reinterpret_cast<float2*>(smem_raw + SM::X1);
   float2* tw = reinterpret_cast<float2*>(smem_raw + SM::TW);
   const int tid = threadIdx.x;
+  // In this order: the unfold kernel's early CTAs, and the voltage-peak kernel, read the caller's arrays and
+  // the tables and write the reconstruction's state without a wait of their own. What an earlier kernel wrote
+  // there is complete because they start only after every CTA here has waited for that kernel.
   if (prm.wait_first) pdl_wait_prior();
   pdl_launch_dependents();
   // threads [0, T) transform (their barriers are named barrier 1); a ninth warp, if there is one, forms
