@@ -1134,10 +1134,13 @@ cudaError_t launch_gemm(ar_ctx* ctx, __nv_bfloat16* const (&a)[3], size_t m_pad,
   const int groups = gemm_groups(m_pad, which, ctx->num_sms);
   if (groups > 1) post = nullptr;
   gp.chunks_per_group = gp.chunks / groups;
-  // 256-wide tiles when every item is a single fold unit and at least two tiles per SM remain. At width 128
-  // an MMA's operands (8 KB in 64 cycles) take all of shared memory's bandwidth and the stages' copies
-  // slow it; at 256 (12 KB in 128) there is room for them: x6 at 43 x 29 pairs of 4096 samples 125.2 ->
-  // 119.3 us the call, at 124 x 64 of 2048 288.0 -> 265.4.
+  // 256-wide tiles when every item is a single fold unit and, for the kernel that stores D, at least two
+  // tiles per SM remain. At width 128 an MMA's operands (8 KB in 64 cycles) take all of shared memory's
+  // bandwidth and the stages' copies slow it; at 256 (12 KB in 128) there is room for them: x6 at 43 x 29 pairs
+  // of 4096 samples 125.2 -> 119.3 us the call, at 124 x 64 of 2048 288.0 -> 265.4. The kernel with the post-pass
+  // has wide tiles only, wherever K is not split: with 152 SMs from 2560 rows, 80 tiles, on. It is the faster one
+  // there too: 17 x 9 pairs of 4096 samples x3 44.1 -> 40.2 us, x6 47.3 -> 44.3; 34 x 9 of 2048 41.1 -> 38.5,
+  // 43.2 -> 42.4; 36 x 17 of 1024 40.6 -> 35.6, 42.9 -> 38.8.
   const bool wide = post || (gp.chunks_per_group <= tc::kFoldChunks && n % 256 == 0 &&
                              static_cast<long long>(m_pad / tc::kBM) * (n / 256) >= 2 * ctx->num_sms);
   const int bn = wide ? 256 : tc::kBN;
