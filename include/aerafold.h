@@ -244,7 +244,10 @@ ar_status ar_kernel_times(ar_ctx* ctx, float* ms);
  * to 2^-24 (FP32-level). Interpolation, solve, twiddles and the sub-block-phase DFTs are FP32
  * as in ar_unfold; direction cells and timing FP64. The library keeps a workspace of about
  * 20 B per station sample and up to 2^25 x 10 B for the pairs (processed in chunks of
- * 2^25 / N pairs).
+ * 2^25 / N pairs). A context's first call builds its DFT operands on the host and allocates their device
+ * copies and the workspace, synchronously: about 26 ms, 200 times a later call (43 x 29 pairs of 4096
+ * samples); ar_prepare does not cover it, and a call that needs a larger workspace allocates again. Make that
+ * call ahead of a time-critical section or a stream capture.
  * ev, out: as ar_unfold (device memory); S * N <= 2^24.
  * With ar_set_profiling on, ar_kernel_times gives ms[0] = forward transform and the first
  * chunk's solve, ms[1] = the first chunk's inverse GEMM (with the post-pass, unless sub-sample times,
